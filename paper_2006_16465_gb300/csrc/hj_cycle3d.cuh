@@ -86,6 +86,21 @@ __device__ __forceinline__ T point_update3(const Coef3<T> &k, T g, T W, T E, T S
     }
 }
 
+// Binary64 update from the rounded products of the six neighbours (the order of
+// point_update3; see update_from_products).
+template <typename T, bool WANT_RES>
+__device__ __forceinline__ T update3_from_products(const Coef3<T> &k, T g, T pW, T pE, T pS, T pN, T pB, T pT, T old,
+                                                   T &res) {
+    double acc = __dadd_rn(pW, pE);
+    acc = __dadd_rn(acc, pS);
+    acc = __dadd_rn(acc, pN);
+    acc = __dadd_rn(acc, pB);
+    acc = __dadd_rn(acc, pT);
+    const double t = __dsub_rn(g, acc);
+    if constexpr (WANT_RES) res = (T)__dsub_rn(t, __dmul_rn(k.dconst, old));
+    return (T)__dmul_rn(t, k.invd);
+}
+
 template <typename S, typename T, int LX, int RY, int RZ, int NW, bool EXACT, bool RES>
 __global__ void __launch_bounds__(32 * NW) hier3d_kernel(const CycArgs a) {
     constexpr int LY = 32 / LX, TX = LX, TY = LY * RY, TZ = RZ;
@@ -166,44 +181,90 @@ __global__ void __launch_bounds__(32 * NW) hier3d_kernel(const CycArgs a) {
                 hT[r] = ld_u(x, yl + r, z0 + TZ);
             }
         }
-        for (int s = 0; s < a.k; ++s) {
-            T prev[RY];   // old values of the plane below
+        // SYM (binary64): the neighbours share the products c u_p as in 2D
+        // (update_from_products): 1 with W = E, S = N and B = T (13 operations a
+        // point become 10), 2 with all six equal (8).  The halo registers then
+        // hold products, u holds values.
+        auto run = [&](auto sym_tag) {
+            constexpr int SYM = decltype(sym_tag)::value;
+            auto mul = [](T c, T v) -> T {
+                if constexpr (SYM != 0) return (T)__dmul_rn(c, v);
+                else return v;
+            };
+            if constexpr (SYM != 0) {
 #pragma unroll
-            for (int r = 0; r < RY; ++r) prev[r] = hB[r];
+                for (int z = 0; z < RZ; ++z) {
 #pragma unroll
-            for (int z = 0; z < RZ; ++z) {
-                T up = sS[z], dn = sN[z];
-                if constexpr (LY > 1) {
-                    const T a_up = __shfl_up_sync(FULL, u[RY - 1][z], LX);
-                    const T a_dn = __shfl_down_sync(FULL, u[0][z], LX);
-                    if (gy > 0) up = a_up;
-                    if (gy < LY - 1) dn = a_dn;
-                }
-                T nv[RY];
-#pragma unroll
-                for (int r = 0; r < RY; ++r) {
-                    const T c = u[r][z];
-                    T Wv = __shfl_up_sync(FULL, c, 1, LX);
-                    T Ev = __shfl_down_sync(FULL, c, 1, LX);
-                    if (lx == 0) Wv = xh[r][z];
-                    if (lx == LX - 1) Ev = xh[r][z];
-                    const T Sv = r > 0 ? u[r - 1][z] : up;
-                    const T Nv = r < RY - 1 ? u[r + 1][z] : dn;
-                    const T Tv = z < RZ - 1 ? u[r][z + 1] : hT[r];
-                    T res = 0;
-                    const T v = point_update3<T, EXACT, RES>(kc, g[r][z], Wv, Ev, Sv, Nv, prev[r], Tv, c, res);
-                    const bool in = full || (x <= nx && yl + r <= ny && z0 + z <= nz);
-                    nv[r] = in ? v : c;
-                    if constexpr (RES) {
-                        if (s == 0 && in) acc += (Acc)res * (Acc)res;
-                    }
+                    for (int r = 0; r < RY; ++r) xh[r][z] = mul(kc.cW, xh[r][z]);
+                    sS[z] = mul(kc.cS, sS[z]);
+                    sN[z] = mul(kc.cS, sN[z]);
                 }
 #pragma unroll
                 for (int r = 0; r < RY; ++r) {
-                    prev[r] = u[r][z];
-                    u[r][z] = nv[r];
+                    hB[r] = mul(kc.cB, hB[r]);
+                    hT[r] = mul(kc.cB, hT[r]);
                 }
             }
+            for (int s = 0; s < a.k; ++s) {
+                T prev[RY], mid[RY];   // B terms of the plane, and the plane's own z terms
+#pragma unroll
+                for (int r = 0; r < RY; ++r) {
+                    prev[r] = hB[r];
+                    mid[r] = mul(kc.cB, u[r][0]);
+                }
+#pragma unroll
+                for (int z = 0; z < RZ; ++z) {
+                    T ty[RY], nxt[RY];   // the plane's y terms, the T terms
+#pragma unroll
+                    for (int r = 0; r < RY; ++r) {
+                        ty[r] = SYM == 2 ? mid[r] : mul(kc.cS, u[r][z]);
+                        nxt[r] = z < RZ - 1 ? mul(kc.cB, u[r][z < RZ - 1 ? z + 1 : 0]) : hT[r];
+                    }
+                    T up = sS[z], dn = sN[z];
+                    if constexpr (LY > 1) {
+                        const T a_up = __shfl_up_sync(FULL, ty[RY - 1], LX);
+                        const T a_dn = __shfl_down_sync(FULL, ty[0], LX);
+                        if (gy > 0) up = a_up;
+                        if (gy < LY - 1) dn = a_dn;
+                    }
+                    T nv[RY];
+#pragma unroll
+                    for (int r = 0; r < RY; ++r) {
+                        const T c = u[r][z];
+                        const T tx = SYM == 2 ? mid[r] : mul(kc.cW, c);
+                        T Wv = __shfl_up_sync(FULL, tx, 1, LX);
+                        T Ev = __shfl_down_sync(FULL, tx, 1, LX);
+                        if (lx == 0) Wv = xh[r][z];
+                        if (lx == LX - 1) Ev = xh[r][z];
+                        const T Sv = r > 0 ? ty[r > 0 ? r - 1 : 0] : up;
+                        const T Nv = r < RY - 1 ? ty[r < RY - 1 ? r + 1 : 0] : dn;
+                        T res = 0, v;
+                        if constexpr (SYM != 0)
+                            v = update3_from_products<T, RES>(kc, g[r][z], Wv, Ev, Sv, Nv, prev[r], nxt[r], c, res);
+                        else
+                            v = point_update3<T, EXACT, RES>(kc, g[r][z], Wv, Ev, Sv, Nv, prev[r], nxt[r], c, res);
+                        const bool in = full || (x <= nx && yl + r <= ny && z0 + z <= nz);
+                        nv[r] = in ? v : c;
+                        if constexpr (RES) {
+                            if (s == 0 && in) acc += (Acc)res * (Acc)res;
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < RY; ++r) {
+                        prev[r] = mid[r];
+                        mid[r] = nxt[r];
+                        u[r][z] = nv[r];
+                    }
+                }
+            }
+        };
+        if constexpr (EXACT) {
+            const bool pairs = same_bits(kc.cW, kc.cE) && same_bits(kc.cS, kc.cN) && same_bits(kc.cB, kc.cT);
+            if (pairs && same_bits(kc.cW, kc.cS) && same_bits(kc.cW, kc.cB)) run(std::integral_constant<int, 2>());
+            else if (pairs) run(std::integral_constant<int, 1>());
+            else run(std::integral_constant<int, 0>());
+        } else {
+            run(std::integral_constant<int, 0>());
         }
         // write back this lane's interior points
         S *uo = (S *)a.uout;

@@ -210,51 +210,81 @@ __global__ void __launch_bounds__(1024 / RPT, (RPT == 1 && STAGE == MG_PLAIN) ? 
     }
     const T hs = ty == 0 ? ld_u(j0 - 1, i) : (T)0;
     const T hn = ty == BY - 1 ? ld_u(j0 + TY, i) : (T)0;
-#pragma unroll
-    for (int m = 0; m < RPT; ++m) {
-        const int me = (ty + m * BY + 1) * lw + tx + 1;
-        buf0[me] = v0[m];
-        buf1[me] = v0[m];
-        if (tx == 0) { buf0[me - 1] = hw[m]; buf1[me - 1] = hw[m]; }
-        if (tx == TX - 1) { buf0[me + 1] = he[m]; buf1[me + 1] = he[m]; }
-    }
-    if (ty == 0) { buf0[tx + 1] = hs; buf1[tx + 1] = hs; }
-    if (ty == BY - 1) { buf0[(TY + 1) * lw + tx + 1] = hn; buf1[(TY + 1) * lw + tx + 1] = hn; }
-    __syncthreads();
-    for (int s = 0; s < a.k; ++s) {
-        const T *src = (s & 1) ? buf1 : buf0;
-        T *dst = (s & 1) ? buf0 : buf1;
+    // Binary64 with four equal coefficients: the containers hold the products
+    // c u_p, each formed once by its point's thread instead of once per
+    // neighbour, and a thread keeps its own values in registers (12 FP64
+    // operations a point and subiteration become 9, every rounding unchanged;
+    // the FP64 pipe bounds this kernel, see update_from_products; 1023 x 1023 to
+    // 1e-8: 5.94 -> 5.30 ms).  Otherwise they hold the values.
+    bool share = false;
+    if constexpr (EXACT) share = same_bits(a.cW, a.cE) && same_bits(a.cS, a.cN) && same_bits(a.cW, a.cS);
+    auto run = [&](auto share_tag) {
+        constexpr bool SH = decltype(share_tag)::value;
+        auto term = [&](T v) -> T {
+            if constexpr (SH) return (T)__dmul_rn(a.cW, v);
+            else return v;
+        };
 #pragma unroll
         for (int m = 0; m < RPT; ++m) {
-            if (!in[m]) continue;
             const int me = (ty + m * BY + 1) * lw + tx + 1;
-            const T old = src[me];
-            const T W = src[me - 1], E = src[me + 1], Sv = src[me - lw], Nv = src[me + lw];
-            T nv;
-            if constexpr (EXACT) {
-                double acc = __dmul_rn(a.cW, W);
-                acc = __dadd_rn(acc, __dmul_rn(a.cE, E));
-                acc = __dadd_rn(acc, __dmul_rn(a.cS, Sv));
-                acc = __dadd_rn(acc, __dmul_rn(a.cN, Nv));
-                const double jac = __dmul_rn(__dsub_rn(g[m], acc), a.invd);
-                nv = __dadd_rn(old, __dmul_rn(a.omega, __dsub_rn(jac, old)));
-            } else {
-                T t = g[m];
-                t = fmaf(a.fN, Nv, t);
-                t = fmaf(a.fS, Sv, t);
-                t = fmaf(a.fE, E, t);
-                t = fmaf(a.fW, W, t);
-                nv = fmaf(a.fomega, t - old, old);
-            }
-            dst[me] = nv;
+            const T p0 = term(v0[m]);
+            buf0[me] = p0;
+            buf1[me] = p0;
+            if (tx == 0) { const T w = term(hw[m]); buf0[me - 1] = w; buf1[me - 1] = w; }
+            if (tx == TX - 1) { const T e = term(he[m]); buf0[me + 1] = e; buf1[me + 1] = e; }
         }
+        if (ty == 0) { const T w = term(hs); buf0[tx + 1] = w; buf1[tx + 1] = w; }
+        if (ty == BY - 1) { const T w = term(hn); buf0[(TY + 1) * lw + tx + 1] = w; buf1[(TY + 1) * lw + tx + 1] = w; }
         __syncthreads();
+        for (int s = 0; s < a.k; ++s) {
+            const T *src = (s & 1) ? buf1 : buf0;
+            T *dst = (s & 1) ? buf0 : buf1;
+            const bool more = s + 1 < a.k;   // the last subiteration's values go to global memory from registers
+#pragma unroll
+            for (int m = 0; m < RPT; ++m) {
+                if (!in[m]) continue;
+                const int me = (ty + m * BY + 1) * lw + tx + 1;
+                const T old = v0[m];
+                const T W = src[me - 1], E = src[me + 1], Sv = src[me - lw], Nv = src[me + lw];
+                T nv;
+                if constexpr (EXACT) {
+                    double acc;
+                    if constexpr (SH) {
+                        acc = __dadd_rn(W, E);
+                        acc = __dadd_rn(acc, Sv);
+                        acc = __dadd_rn(acc, Nv);
+                    } else {
+                        acc = __dmul_rn(a.cW, W);
+                        acc = __dadd_rn(acc, __dmul_rn(a.cE, E));
+                        acc = __dadd_rn(acc, __dmul_rn(a.cS, Sv));
+                        acc = __dadd_rn(acc, __dmul_rn(a.cN, Nv));
+                    }
+                    const double jac = __dmul_rn(__dsub_rn(g[m], acc), a.invd);
+                    nv = __dadd_rn(old, __dmul_rn(a.omega, __dsub_rn(jac, old)));
+                } else {
+                    T t = g[m];
+                    t = fmaf(a.fN, Nv, t);
+                    t = fmaf(a.fS, Sv, t);
+                    t = fmaf(a.fE, E, t);
+                    t = fmaf(a.fW, W, t);
+                    nv = fmaf(a.fomega, t - old, old);
+                }
+                v0[m] = nv;
+                if (more) dst[me] = term(nv);
+            }
+            if (more) __syncthreads();
+        }
+    };
+    if constexpr (EXACT) {
+        if (share) run(std::integral_constant<bool, true>());
+        else run(std::integral_constant<bool, false>());
+    } else {
+        run(std::integral_constant<bool, false>());
     }
-    const T *fin = (a.k & 1) ? buf1 : buf0;
 #pragma unroll
     for (int m = 0; m < RPT; ++m) {
         const int j = j0 + ty + m * BY;
-        if (in[m]) ((T *)a.uout)[(long long)j * ld + i] = fin[(ty + m * BY + 1) * lw + tx + 1];
+        if (in[m]) ((T *)a.uout)[(long long)j * ld + i] = v0[m];
     }
 }
 

@@ -1,0 +1,64 @@
+"""Binary64 kernels share a neighbour's product c u between the points that read
+it where coefficients are equal: none shared (general stencil), opposite pairs
+equal (rectangular grid), all equal (square grid, cube).  Every rounding stays
+where the general path has it, so the cycles equal the oracle's bit for bit in
+each mode, on ragged grids and with a screening field."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+from helpers import gpu_solver, rel_max, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def _cycles(p, dim, **kw):
+    import torch
+    s = gpu_solver(p, precision="f64", **kw)
+    u = to_dev(p.u0, dim, torch.float64)
+    s.solve(to_dev(p.f, dim, torch.float64), u)
+    s.close()
+    return to_host(u, p.st.nx)
+
+
+@pytest.mark.parametrize("engine", [dict(pipeline=0), dict(pipeline=1), dict(pipeline=0, overlap_x=4, overlap_y=6)])
+@pytest.mark.parametrize("shape,sigma,asym", [((71, 71), "field", False), ((71, 71), "none", False),
+                                               ((71, 38), "field", False), ((71, 71), "none", True)])
+def test_2d_modes(shape, sigma, asym, engine):
+    import paper_2006_16465_gb300 as hj
+    p = W.random_bc_problem(2, *shape, seed=shape[1], sigma_kind=sigma, asym=asym)
+    ovl = (engine.get("overlap_x", 0), engine.get("overlap_y", 0))
+    for tx, ty, th in hj.hj_tile_variants(2, hj.PRECISIONS["f64"]):
+        if max(ovl) and (ty <= max(ovl) or tx <= max(ovl)):
+            continue
+        got = _cycles(p, 2, tile_x=tx, tile_y=ty, tile_threads=th, k=3, fixed_cycles=3, **engine)
+        ref = oracle.run_fixed(p.st, p.f, p.u0, 3, tx, ty, 3, overlap=ovl)
+        assert np.array_equal(got, ref), (tx, ty, th, rel_max(got, ref))
+
+
+@pytest.mark.parametrize("shape,asym", [((19, 19, 19), False), ((33, 33, 20), False), ((33, 20, 9), True)])
+def test_3d_modes(shape, asym):
+    import paper_2006_16465_gb300 as hj
+    p = W.random_bc_problem3d(*shape, seed=sum(shape), sigma_kind="const", asym=asym)
+    for tx, ty, tz in hj.hj_tile_shapes3d(hj.PRECISIONS["f64"]):
+        got = _cycles(p, 3, tile_x=tx, tile_y=ty, tile_z=tz, k=3, fixed_cycles=2)
+        ref = oracle.run_fixed(p.st, p.f, p.u0, 2, tx, ty, 3, tz=tz)
+        assert np.array_equal(got, ref), (tx, ty, tz, rel_max(got, ref))
+
+
+@pytest.mark.parametrize("shape,tile", [((63, 63), (32, 8)), ((63, 63), (16, 2)), ((95, 95), (8, 3)), ((63, 31), (32, 8))])
+def test_multigrid_modes(shape, tile):
+    p = W.random_bc_problem(2, *shape, seed=9, sigma_kind="const")
+    L = oracle.mg_max_levels(*shape)
+    got = _cycles(p, 2, method="mg", tile_x=tile[0], tile_y=tile[1], k=3, fixed_cycles=2)
+    ref = p.u0
+    for _ in range(2):
+        ref = oracle.mg_vcycle(p.st, p.f, ref, L, 1, 1, tile[0], tile[1], 3, 0.8)
+    assert np.array_equal(got, ref), rel_max(got, ref)
