@@ -233,6 +233,7 @@ RedArgs red_args(const hj_handle *h, int mode, double tol, long long max_cycles)
     r.out = h->rstore;
     r.ctl = h->ctl;
     r.tol = tol;
+    r.tol2 = tol * tol * (1.0 + 1e-9);
     r.max_cycles = max_cycles;
     r.mode = mode;
     r.scale = 1.0;
@@ -328,9 +329,11 @@ struct Plan {
 };
 
 // Largest grid of the one-CTA-per-subdomain kernels that folds its residual
-// in the next launch (one warp sums one partial per CTA; larger grids keep the
-// grid reduction at the launch's end).
-constexpr long long kDeferMaxBlocks = 4096;
+// in the next launch.  A CTA of its own folds while the others sweep, in less
+// time than they take at any size: 65,536 partials (8192 x 8192 in 32 x 32
+// subdomains) are about 40 us of loads and adds against launches of 130 us
+// (binary32) and more.  Beyond that the grid reduction at the launch's end stays.
+constexpr long long kDeferMaxBlocks = 65536;
 
 // 3D: whether the prefetching (persistent-warp, cp.async) kernel runs.  Only
 // on request (pipeline = 1): measured at 512^3 binary32 it is slower than the
@@ -408,12 +411,12 @@ bool want_ppc(const hj_handle *h, const PpcKernelInfo *pi, bool classic) {
     return ntiles >= 8LL * h->nsm;
 }
 
-// Whether a converging run of the one-CTA-per-subdomain 2D kernels folds its
-// residual in the next launch (as the pipelined kernel always does): 2D
+// Whether a converging run of the one-CTA-per-subdomain kernels folds its
+// residual in the next launch (as the pipelined kernel always does): 1D and 2D
 // hierarchical cycles with constant coefficients on grids of at most
-// kDeferMaxBlocks subdomains.
+// kDeferMaxBlocks CTAs.
 bool defer_hier(const hj_handle *h, const TileKernelInfo *ki, bool classic) {
-    if (classic || !ki || h->d.dim != 2 || h->d.coef) return false;
+    if (classic || !ki || h->d.dim == 3 || h->d.coef) return false;
     dim3 g, b;
     geometry(h, ki, false, &g, &b);
     return (long long)g.x * g.y <= kDeferMaxBlocks;
@@ -538,7 +541,9 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
             // deferred fold: launch c reads B[c % 3], writes B[(c+1) % 3] and
             // its per-CTA partials to slot c % 2, folded by launch c + 1
             if (!b2) return seterr(HJ_ERR_CUDA, "internal: deferred residual runs need a third iterate buffer");
+            // (the reduction workspace holds two slots of one partial per subdomain)
             const long long nb = (long long)pl->grid.x * pl->grid.y;
+            pl->grid = dim3((unsigned)nb + 1);   // CTA 0 folds, CTA 1 + t sweeps subdomain t
             CKS(ensure_reduction(h, (size_t)nb));
             void *bufs[3] = {b0, b1, b2};
             pl->deferred = true;
@@ -814,7 +819,13 @@ int iterate(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int
             if (blocks > 64LL * cap) return seterr(HJ_ERR_UNSUPPORTED, "grid too large for the persistent engine");
             use = true;
         } else {
-            use = blocks <= cap;
+            // hierarchical cycles run as graphs of launches: a kernel boundary
+            // inside a graph costs 1.0 us on this part, a grid barrier 1.5 to 2.5
+            // us and the decision behind it another 1.5, where the graph's fold
+            // runs beside the sweeps (32 x 32, k = 32, binary32 cycles:
+            // 512 x 512 10.1 against 6.4 us a cycle, 64 x 64 8.8 against 6.5; 1D
+            // binary64, 512 points 12.3 against 10.2)
+            use = pclassic && blocks <= cap;
         }
     }
     if (used_persistent) *used_persistent = use ? 1 : 0;

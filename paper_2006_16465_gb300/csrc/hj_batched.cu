@@ -604,6 +604,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         q.a.uout = b.dB;
         q.a.dinv = b.dinv;
         q.a.red.tol = par.inner_tol;
+        q.a.red.tol2 = par.inner_tol * par.inner_tol * (1.0 + 1e-9);
         q.a.red.max_cycles = par.inner_max_cycles;
         // the per-point-diagonal kernel forms r itself; the constant-diagonal one forms (u' - u)
         q.a.red.scale = sig_any ? 1.0 : q.a.dconst * q.a.dconst;

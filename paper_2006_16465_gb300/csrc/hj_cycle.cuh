@@ -725,14 +725,21 @@ __device__ __forceinline__ void store2d(const Tile2D<T, C, R, SIG> &t, const Cyc
     }
 }
 
+// stop (nullable): set where the run has already ended; read with the staging
+// loads in flight, it ends the CTA before the sweeps (nothing is written).
 template <typename S, typename T, int C, int R, int NW, int H, bool EXACT, bool SIG, bool RES, bool PART,
           bool OVL = false>
 __device__ __forceinline__ typename std::conditional<EXACT, double, T>::type
-tile2d(const CycArgs &a, const int x0, const int y0, T *xbuf, const Own own = Own{0, 0, 0, 0}) {
+tile2d(const CycArgs &a, const int x0, const int y0, T *xbuf, const Own own = Own{0, 0, 0, 0},
+       const int *stop = nullptr) {
     const int yb = y0 + band_of_lane<R, H>() * R;
     const Coef<T> kc = make_coef<T>(a);
     Tile2D<T, C, R, SIG> t;
     stage2d_global<S, T, C, R, H, EXACT, SIG, PART>(t, a, kc, x0, yb);
+    if (stop) {
+        // one answer for the whole CTA: this launch's fold may be setting the flag now
+        if (NW == 1 ? __any_sync(FULL, *stop) : __syncthreads_or(*stop)) return 0;
+    }
     auto acc = sweeps2d<T, C, R, NW, H, EXACT, SIG, RES, PART, OVL>(t, kc, a.k, x0, yb, a.nx, a.ny, xbuf, own, a.dbg);
     store2d<S, T, C, R, H, SIG, PART, OVL>(t, a, x0, yb, own);
     return acc;
@@ -762,42 +769,51 @@ __device__ __forceinline__ void write_cta_partial(double *slot, A acc) {
 
 // OVL: overlapping subdomains (Sections 3.4, 4.3): block (bx, by) is subdomain
 // (bx, by) of a.jx x a.jy, placed and owning points as subdomain_span says.
-// RES with a.part_w set: the deferred fold (one partial per CTA, folded by the
-// next launch's last CTA) instead of the grid reduction at the launch's end.
+// RES with a.part_w set: the deferred fold.  The grid is then 1 + a.jx a.jy CTAs
+// in a row: CTA 1 + t sweeps subdomain t and writes one partial, and CTA 0 folds
+// the previous launch's partials while they sweep.  (With the fold in front of
+// the last subdomain's sweeps, it was the launch's critical path on small
+// grids: 4 to 5 us of a 14 us cycle of k = 64 on 512 x 512.)  The flags that end
+// a run are read beside the staging loads, not before them.
 template <typename S, typename T, int C, int R, int NW, int H, bool EXACT, bool SIG, bool RES, bool OVL = false>
 __global__ void __launch_bounds__(32 * NW) hier2d_kernel(const CycArgs a) {
-    const int nblk = (int)(gridDim.x * gridDim.y), bid = (int)(blockIdx.y * gridDim.x + blockIdx.x);
+    int bx = blockIdx.x, by = blockIdx.y, stop = 0, tile = 0;
     if constexpr (RES) {
         volatile Ctl *ctl = a.red.ctl;
-        if (ctl->done >= 0) return;
         if (a.part_w) {
-            const bool reducer = bid == nblk - 1;
-            if (ctl->fold_only[a.parity]) {
-                if (reducer && threadIdx.x < 32) deferred_fold_parts(a.red, a.part_r, nblk, a.parity);
+            if (blockIdx.x == 0) {
+                if (ctl->done < 0) deferred_fold_parts<NW>(a.red, a.part_r, (int)gridDim.x - 1, a.parity);
                 return;
             }
-            if (reducer && threadIdx.x < 32) deferred_fold_parts(a.red, a.part_r, nblk, a.parity);
+            tile = (int)blockIdx.x - 1;
+            by = tile / a.jx;
+            bx = tile - by * a.jx;
+            stop = (ctl->done >= 0) | ctl->fold_only[a.parity];
+        } else {
+            stop = ctl->done >= 0;
         }
     }
     constexpr int TX = 32 * C / H, TY = R * NW * H;
     constexpr int XB = NW > 1 ? 2 * NW * 2 * TX : 1;
     __shared__ T xbuf[XB];
-    int x0 = 1 + blockIdx.x * TX, y0 = 1 + blockIdx.y * TY;
+    int x0 = 1 + bx * TX, y0 = 1 + by * TY;
     Own own{0, 0, 0, 0};
     if constexpr (OVL) {
-        const Span sx = subdomain_span(blockIdx.x, a.jx, a.nx, TX, a.ox);
-        const Span sy = subdomain_span(blockIdx.y, a.jy, a.ny, TY, a.oy);
+        const Span sx = subdomain_span(bx, a.jx, a.nx, TX, a.ox);
+        const Span sy = subdomain_span(by, a.jy, a.ny, TY, a.oy);
         x0 = sx.start;
         y0 = sy.start;
         own = Own{sx.lo, sx.hi, sy.lo, sy.hi};
     }
     const bool full = (x0 + TX - 1 <= a.nx) && (y0 + TY - 1 <= a.ny);
     typename std::conditional<EXACT, double, T>::type acc;
-    if (full) acc = tile2d<S, T, C, R, NW, H, EXACT, SIG, RES, false, OVL>(a, x0, y0, xbuf, own);
-    else acc = tile2d<S, T, C, R, NW, H, EXACT, SIG, RES, true, OVL>(a, x0, y0, xbuf, own);
+    if (full) acc = tile2d<S, T, C, R, NW, H, EXACT, SIG, RES, false, OVL>(a, x0, y0, xbuf, own, RES ? &stop : nullptr);
+    else acc = tile2d<S, T, C, R, NW, H, EXACT, SIG, RES, true, OVL>(a, x0, y0, xbuf, own, RES ? &stop : nullptr);
     if constexpr (RES) {
-        if (a.part_w) write_cta_partial<NW>(a.part_w + bid, acc);
-        else reduce_grid_acc(a.red, acc);
+        // (a stopped CTA's partial and reduction share are never read: the run's
+        // answer stands, and the next solve resets the control block)
+        if (a.part_w) write_cta_partial<NW>(a.part_w + tile, acc);
+        else if (!stop) reduce_grid_acc(a.red, acc);
     }
 }
 
@@ -818,7 +834,8 @@ struct Xchg1D {
 
 template <typename S, typename T, int C, int WPT, bool EXACT, bool SIG, bool RES, bool PART, bool OVL = false>
 __device__ __forceinline__ typename std::conditional<EXACT, double, T>::type
-tile1d(const CycArgs &a, const int x0, const int row, Xchg1D<T, WPT> &xb, const int own_lo = 0, const int own_hi = 0) {
+tile1d(const CycArgs &a, const int x0, const int row, Xchg1D<T, WPT> &xb, const int own_lo = 0, const int own_hi = 0,
+       const int *stop = nullptr) {
     constexpr int TX = 32 * C * WPT;
     const int lane = threadIdx.x & 31, q = (threadIdx.x >> 5) % WPT;
     const int xl = x0 + q * 32 * C + lane * C;
@@ -851,6 +868,11 @@ tile1d(const CycArgs &a, const int x0, const int row, Xchg1D<T, WPT> &xb, const 
     const int hcol = wl ? x0 - 1 : x0 + TX;
     const bool hok = (wl || el) && (!PART || hcol <= nx + 1) && HJ_IN(a.dbg, rb + hcol, grid_elems1d(a), 32);
     const T hx = hok ? ld_s<S, T>(uin + rb + hcol) : (T)0;
+    // the run has already ended (read beside the loads above, one answer per CTA
+    // where warps meet at barriers)
+    if (stop) {
+        if (WPT == 1 ? __any_sync(FULL, *stop) : __syncthreads_or(*stop)) return 0;
+    }
 
     typedef typename std::conditional<EXACT, double, T>::type Acc;
     Acc acc = 0;
@@ -927,12 +949,27 @@ tile1d(const CycArgs &a, const int x0, const int row, Xchg1D<T, WPT> &xb, const 
 template <typename S, typename T, int C, int WPT, int WPB, bool EXACT, bool SIG, bool RES, bool OVL = false>
 __global__ void __launch_bounds__(32 * WPT * WPB) hier1d_kernel(const CycArgs a) {
     static_assert(WPT == 1 || WPB == 1, "several subdomains per CTA only with one warp each");
+    int bx = blockIdx.x, row = blockIdx.y, stop = 0, blk = 0;
     if constexpr (RES) {
-        if (*(volatile int *)&a.red.ctl->done >= 0) return;
+        volatile Ctl *ctl = a.red.ctl;
+        if (a.part_w) {
+            // deferred fold, as in hier2d_kernel: CTA 0 folds the previous launch's partials
+            if (blockIdx.x == 0) {
+                if (ctl->done < 0) deferred_fold_parts<WPT * WPB>(a.red, a.part_r, (int)gridDim.x - 1, a.parity);
+                return;
+            }
+            blk = (int)blockIdx.x - 1;
+            const int gx = (a.jx + WPB - 1) / WPB;
+            row = blk / gx;
+            bx = blk - row * gx;
+            stop = (ctl->done >= 0) | ctl->fold_only[a.parity];
+        } else {
+            stop = ctl->done >= 0;
+        }
     }
     constexpr int TX = 32 * C * WPT;
     __shared__ Xchg1D<T, WPT> xb;
-    const int j = blockIdx.x * WPB + (int)(threadIdx.x >> 5) / WPT;   // subdomain along the row
+    const int j = bx * WPB + (int)(threadIdx.x >> 5) / WPT;   // subdomain along the row
     int x0 = 1 + j * TX, lo = 0, hi = 0;
     bool here = x0 <= a.nx;
     if constexpr (OVL) {
@@ -944,15 +981,18 @@ __global__ void __launch_bounds__(32 * WPT * WPB) hier1d_kernel(const CycArgs a)
             hi = sp.hi;
         }
     }
-    const int row = blockIdx.y;
     typename std::conditional<EXACT, double, T>::type acc = 0;
     // with WPT > 1, the subdomain is uniform across the CTA and the whole CTA
     // takes the same branch; with WPB > 1 the branches hold no barrier
+    const int *sp = RES ? &stop : nullptr;
     if (here) {
-        if (x0 + TX - 1 <= a.nx) acc = tile1d<S, T, C, WPT, EXACT, SIG, RES, false, OVL>(a, x0, row, xb, lo, hi);
-        else acc = tile1d<S, T, C, WPT, EXACT, SIG, RES, true, OVL>(a, x0, row, xb, lo, hi);
+        if (x0 + TX - 1 <= a.nx) acc = tile1d<S, T, C, WPT, EXACT, SIG, RES, false, OVL>(a, x0, row, xb, lo, hi, sp);
+        else acc = tile1d<S, T, C, WPT, EXACT, SIG, RES, true, OVL>(a, x0, row, xb, lo, hi, sp);
     }
-    if constexpr (RES) reduce_grid_acc(a.red, acc);
+    if constexpr (RES) {
+        if (a.part_w) write_cta_partial<WPT * WPB>(a.part_w + blk, acc);
+        else if (!stop) reduce_grid_acc(a.red, acc);
+    }
 }
 
 // ---------------------------------------------------------------------------

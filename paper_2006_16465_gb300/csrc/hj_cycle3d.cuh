@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcAr
         volatile Ctl *ctl = a.red.ctl;
         if (ctl->done >= 0) return;
         if (ctl->fold_only[P.parity]) {
-            if (reducer) deferred_fold(P);
+            if (reducer) deferred_fold<1>(P);
             return;
         }
     }
@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcAr
     // the last CTA has the fewest subdomains when the grid does not divide
     // them: it folds the previous launch's residual while its first copy lands
     if constexpr (RES) {
-        if (reducer) deferred_fold(P);
+        if (reducer) deferred_fold<1>(P);
     }
     const Coef3<float> kc = make_coef3<float>(a);
     const long long ld = a.ld, ps = a.ps;

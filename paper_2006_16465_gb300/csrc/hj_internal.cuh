@@ -49,6 +49,7 @@ struct RedArgs {
     double *out;         // RED_STORE: NV results
     Ctl *ctl;            // RED_CYCLE: control block
     double tol;          // stop at ||r_c|| <= tol ||r_0||
+    double tol2;         // tol^2 (1 + 1e-9): above tol2 ||r_0||^2 the test fails for sure (0: always test in full)
     double scale;        // RED_CYCLE: the reduced sum is multiplied by this (d^2 for the fast path)
     long long stall_window;  // > 0: also stop when ||r|| moved by <= stall_rtol relative over this many cycles
     double stall_rtol;
@@ -221,19 +222,33 @@ __device__ __forceinline__ bool stalled(const RedArgs &r, long long c, double re
     return fabs(a - b) <= r.stall_rtol * a;
 }
 
+// The stopping test ||r_c|| <= tol ||r_0|| on the squares.  The square roots of
+// the test as stated cost some 3000 clocks on this part's FP64 pipe, on the
+// critical path of every cycle of a small grid, so a margin far wider than
+// their rounding decides first, by comparing bit patterns (positive binary64
+// numbers order like their integers); only within it are they taken.
+__device__ __forceinline__ bool met_tolerance(const RedArgs &r, double res2, double res2_0) {
+    const long long lim = __double_as_longlong(r.tol2 * res2_0);
+    // 2^-962 (1e-290): below it products of subnormals would lose the margin
+    if (lim > (61LL << 52) && lim < 0x7ff0000000000000LL && __double_as_longlong(res2) > lim) return false;
+    return sqrt(res2) <= r.tol * sqrt(res2_0);
+}
+__device__ __forceinline__ bool finite_bits(double x) {
+    return (__double_as_longlong(x) & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
+}
+
 // Fold ||r_c||^2 of the cycle into the control block (runs on one thread).
 __device__ __forceinline__ void finish_cycle(const RedArgs &r, double res2) {
     volatile Ctl *ctl = r.ctl;   // written by earlier launches: bypass L1
     const long long c = ctl->cycle;
+    const double first = ctl->res2_0;
     r.hist[c & (kHistCap - 1)] = res2;
     if (c == 0) ctl->res2_0 = res2;
-    const double r0 = sqrt(c == 0 ? res2 : ctl->res2_0);
-    const double rc = sqrt(res2);
     ctl->res2_last = res2;
-    if (!isfinite(rc)) {
+    if (!finite_bits(res2)) {
         ctl->status = HJ_ERR_DIVERGED;
         ctl->done = (int)c;
-    } else if (rc <= r.tol * r0) {
+    } else if (met_tolerance(r, res2, c == 0 ? res2 : first)) {
         ctl->done = (int)c;
     } else if (stalled(r, c, res2, &ctl->res2_mark, &ctl->mark_cycle)) {
         ctl->done = (int)c;
@@ -320,11 +335,13 @@ __device__ __forceinline__ void reduce_grid(const RedArgs &r, const double (&val
     }
 }
 
-// Deferred fold: one warp sums n per-CTA partials written by the previous
-// launch (fixed order: lane-strided, four interleaved accumulators, then the
-// butterfly) and folds ||r||^2 into the control block.  The kernel boundary
-// orders those writes before these loads; __ldcg skips stale L1 lines.
-__device__ __forceinline__ void fold_partials(const RedArgs &r, const double *part, int n) {
+// Deferred fold: sum n per-CTA partials written by the previous launch in a
+// fixed order: lane-strided, four interleaved accumulators, then the butterfly.
+// A CTA of four or more warps gives each accumulator a warp of its own (the
+// adds of one warp would queue on one sub-partition's FP64 pipe, 64 clocks
+// each); the order, and so the sum, is the same.  The kernel boundary orders
+// the partials' writes before these loads; __ldcg skips stale L1 lines.
+__device__ __forceinline__ double sum_partials(const double *part, int n) {
     const int lane = threadIdx.x & 31;
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
     int b = lane;
@@ -337,21 +354,45 @@ __device__ __forceinline__ void fold_partials(const RedArgs &r, const double *pa
         s3 += x3;
     }
     for (; b < n; b += 32) s0 += __ldcg(part + b);
-    const double s = warp_sum((s0 + s1) + (s2 + s3));
-    if (lane == 0) finish_cycle(r, s * r.scale);
+    return warp_sum((s0 + s1) + (s2 + s3));
+}
+// the same by four warps; the result is warp 0's (whole CTA calls)
+__device__ __forceinline__ double sum_partials_cta4(const double *part, int n) {
+    __shared__ double s_acc[4][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (w < 4) {
+        double s = 0.0;
+        int b = lane;
+        for (; b + 96 < n; b += 128) s += __ldcg(part + b + 32 * w);
+        if (w == 0)
+            for (; b < n; b += 32) s += __ldcg(part + b);
+        s_acc[w][lane] = s;
+    }
+    __syncthreads();
+    if (w != 0) return 0.0;
+    return warp_sum((s_acc[0][lane] + s_acc[1][lane]) + (s_acc[2][lane] + s_acc[3][lane]));
 }
 
-// Deferred fold, run by one warp of the last CTA of a launch: fold the
-// previous launch's partials (nparts of them: the residual of the iterate that
-// launch staged), then decide whether the next launch only folds (its iterate
-// would lie beyond max_cycles).  The launch counter and the flags are touched
-// by this warp only, one launch after another.
+// Deferred fold, run by one CTA of a launch (whole CTA calls; NW = its warps):
+// fold the previous launch's partials (nparts of them: the residual of the
+// iterate that launch staged), then decide whether the next launch only folds
+// (its iterate would lie beyond max_cycles).  The launch counter and the flags
+// are touched by this CTA only, one launch after another.
+template <int NW>
 __device__ __forceinline__ void deferred_fold_parts(const RedArgs &red, const double *part_r, int nparts,
                                                     int parity) {
     volatile Ctl *ctl = red.ctl;
     const long long l = ctl->launch;
-    if (l >= 1) fold_partials(red, part_r, nparts);
-    if ((threadIdx.x & 31) == 0) {
+    double s;
+    // (the first launch finds nothing to fold: what it sums is not used)
+    if constexpr (NW >= 4) {
+        s = sum_partials_cta4(part_r, nparts);
+    } else {
+        if (threadIdx.x >= 32) return;
+        s = sum_partials(part_r, nparts);
+    }
+    if (threadIdx.x == 0) {
+        if (l >= 1) finish_cycle(red, s * red.scale);
         ctl->fold_only[parity ^ 1] = (l + 1 >= red.max_cycles) ? 1 : 0;
         ctl->launch = l + 1;
     }

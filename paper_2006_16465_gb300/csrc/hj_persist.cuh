@@ -242,15 +242,14 @@ __device__ __forceinline__ void retire_check(const PersistArgs &P, int p, int pa
         const double res2 = s * r.scale;
         const long long c = st->cycle;
         if (r.hist) r.hist[c & (kHistCap - 1)] = res2;
+        const double first = st->res2_0;
         if (c == 0) st->res2_0 = res2;
-        const double r0 = sqrt(c == 0 ? res2 : st->res2_0);
-        const double rc = sqrt(res2);
         st->res2_last = res2;
         int retire = 1;
-        if (!isfinite(rc)) {
+        if (!finite_bits(res2)) {
             st->status = HJ_ERR_DIVERGED;
             st->done = (int)c;
-        } else if (rc <= r.tol * r0) {
+        } else if (met_tolerance(r, res2, c == 0 ? res2 : first)) {
             st->done = (int)c;
         } else if (stalled(r, c, res2, &st->res2_mark, &st->mark_cycle)) {
             st->done = (int)c;
@@ -380,12 +379,11 @@ __device__ __forceinline__ bool one_decide(const PersistArgs &P, OneState &ls, i
             const long long c = ls.cycle;
             if (blockIdx.x == 0 && r.hist) r.hist[c & (kHistCap - 1)] = res2;
             if (c == 0) ls.res2_0 = res2;
-            const double r0 = sqrt(ls.res2_0), rc = sqrt(res2);
             ls.res2_last = res2;
-            if (!isfinite(rc)) {
+            if (!finite_bits(res2)) {
                 ls.status = HJ_ERR_DIVERGED;
                 ls.done = (int)c;
-            } else if (rc <= r.tol * r0) {
+            } else if (met_tolerance(r, res2, ls.res2_0)) {
                 ls.done = (int)c;
             } else if (stalled(r, c, res2, &ls.mark, &ls.mark_c)) {
                 ls.done = (int)c;

@@ -103,9 +103,10 @@ struct PpcLayout {
 };
 
 // Deferred fold of the pipelined kernel's residual (deferred_fold_parts over
-// the previous launch's one partial per CTA).
+// the previous launch's one partial per CTA; whole CTA calls).
+template <int NW>
 __device__ __forceinline__ void deferred_fold(const PpcArgs &P) {
-    deferred_fold_parts(P.a.red, P.part_r, (int)gridDim.x, P.parity);
+    deferred_fold_parts<NW>(P.a.red, P.part_r, (int)gridDim.x, P.parity);
 }
 
 template <typename S, typename T, int C, int R, int NW, int H, bool EXACT, bool SIG, bool RES, int NST>
@@ -116,9 +117,11 @@ __global__ void __launch_bounds__(32 * NW) ppc2d_kernel(const __grid_constant__ 
     const bool reducer = blockIdx.x == gridDim.x - 1;
     if constexpr (RES) {
         volatile Ctl *ctl = a.red.ctl;
-        if (ctl->done >= 0) return;
+        // one answer for the whole CTA: the reducer of this launch may be setting done now
+        const int done = ctl->done >= 0;
+        if (NW == 1 ? __any_sync(FULL, done) : __syncthreads_or(done)) return;
         if (ctl->fold_only[P.parity]) {
-            if (reducer && threadIdx.x < 32) deferred_fold(P);
+            if (reducer) deferred_fold<NW>(P);
             return;
         }
     }
@@ -152,7 +155,7 @@ __global__ void __launch_bounds__(32 * NW) ppc2d_kernel(const __grid_constant__ 
     // the last CTA has the fewest tiles when the grid does not divide them:
     // it folds the previous launch's residual while its first copies land
     if constexpr (RES) {
-        if (reducer && tid < 32) deferred_fold(P);
+        if (reducer) deferred_fold<NW>(P);
     }
     const Coef<T> kc = make_coef<T>(a);
     typedef typename std::conditional<EXACT, double, T>::type Acc;
