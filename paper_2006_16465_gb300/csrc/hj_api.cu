@@ -168,6 +168,31 @@ const TileKernelInfo *find_tile(int fam, int dim, int tx, int ty, int threads = 
 
 
 
+// Threads per subdomain of the one-CTA-per-subdomain 2D kernels where the caller
+// leaves the choice (0).  While subdomains are no more than the SMs (twice the
+// SMs), a cycle is the latency of one subdomain's k sweeps, so its rows go to
+// four (two) warps on as many sub-partitions; the values are the same bit for
+// bit.  Binary32, 32 x 32, k = 32, us a cycle with 1, 2, 4 warps: 256 x 256 (64
+// subdomains) 6.21, -, 4.46; 512 x 512 (256) 6.37, 5.52, 5.90; with 8
+// overlapping points and k = 64 (484) 10.2, 10.8, 11.2.  Binary64 (its first
+// variant has four warps, one per sub-partition's FP64 pipe) gains the waits of
+// one warp filled by another: k = 16 with 2, 4, 8 warps: 256 x 256 63, 40, 36;
+// 500 x 300 (160) 87, 77, 75; 900 x 800 (725) 194, 177, 175; 3001 x 2003
+// (5,922) 1352, 1315, 1315.
+int default_threads(int fam, const hj_desc &d, const hj_params &p, int nsm) {
+    if (d.dim != 2 || p.method != HJ_METHOD_HIER || d.coef || p.persistent == 1 || p.pipeline == 1) return 0;
+    const long long n = (long long)subdomain_count(d.nx, p.tile_x, p.overlap_x) *
+                        subdomain_count(d.ny, p.tile_y, p.overlap_y);
+    const int want = fam == FAM_F64 ? (n <= 2LL * nsm ? 256 : 0) : n <= nsm ? 128 : n <= 2LL * nsm ? 64 : 0;
+    int cnt = 0, best = 0;
+    const TileKernelInfo *k = family_tiles(fam, &cnt);
+    for (int i = 0; i < cnt; ++i)
+        if (k[i].dim == 2 && k[i].tx == p.tile_x && k[i].ty == p.tile_y && k[i].threads <= want)
+            best = std::max(best, k[i].threads);
+    const TileKernelInfo *first = find_tile(fam, 2, p.tile_x, p.tile_y);
+    return first && best > first->threads ? best : 0;
+}
+
 double now_ms() {
     return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now().time_since_epoch()).count();
 }
@@ -407,6 +432,11 @@ bool want_ppc(const hj_handle *h, const PpcKernelInfo *pi, bool classic) {
     if (classic || !pi || h->d.dim != 2 || overlapped(h) || h->d.coef) return false;
     if (h->p.pipeline == 1) return true;
     if (h->p.pipeline != -1) return false;
+    // binary64 is bound by the FP64 pipe, not by staging, and CTAs of one
+    // subdomain balance better than static lists of them: 3001 x 2003, 32 x 32,
+    // four warps: k = 1 108 against 114 us a cycle, k = 4 352 against 365,
+    // k = 16 1323 against 1366
+    if (!h->ir && h->fam_outer == FAM_F64) return false;
     const long long ntiles = (long long)((h->d.nx + pi->tx - 1) / pi->tx) * ((h->d.ny + pi->ty - 1) / pi->ty);
     return ntiles >= 8LL * h->nsm;
 }
@@ -1384,7 +1414,8 @@ int hj_create(hj_handle **out, const hj_desc *desc, const hj_params *params) {
     if (d.dim == 3) {
         // kernels picked above (k3) or the classic seven-point sweep
     } else if (ir) {
-        h->k_inner = find_tile(h->fam_inner, d.dim, p.tile_x, p.tile_y, p.tile_threads);
+        const int th = p.tile_threads ? p.tile_threads : default_threads(h->fam_inner, d, p, h->nsm);
+        h->k_inner = find_tile(h->fam_inner, d.dim, p.tile_x, p.tile_y, th);
         if (!h->k_inner)
             HJ_FAIL(HJ_ERR_UNSUPPORTED, "tile %dx%d (%d threads) not built for this precision", p.tile_x, p.tile_y,
                     p.tile_threads);
@@ -1396,7 +1427,8 @@ int hj_create(hj_handle **out, const hj_desc *desc, const hj_params *params) {
     } else {
         // (variable coefficients run their own thread-per-point kernel: any
         // subdomain of at most 1024 points)
-        h->k_outer = d.coef ? nullptr : find_tile(h->fam_outer, d.dim, p.tile_x, p.tile_y, p.tile_threads);
+        const int th = p.tile_threads ? p.tile_threads : default_threads(h->fam_outer, d, p, h->nsm);
+        h->k_outer = d.coef ? nullptr : find_tile(h->fam_outer, d.dim, p.tile_x, p.tile_y, th);
         if (!h->k_outer && !d.coef)
             HJ_FAIL(HJ_ERR_UNSUPPORTED, "tile %dx%d (%d threads) not built for this precision", p.tile_x, p.tile_y,
                     p.tile_threads);

@@ -4,7 +4,9 @@
 namespace hj {
 
 static const TileKernelInfo k_tiles[] = {
-    HJ_K2D(double, double, 1, 16, 2, 1, true),   // 32 x 32
+    HJ_K2D(double, double, 1, 8, 4, 1, true),    // 32 x 32
+    HJ_K2D(double, double, 1, 16, 2, 1, true),   // 32 x 32, two warps
+    HJ_K2D(double, double, 1, 4, 8, 1, true),    // 32 x 32, eight warps
     HJ_K2D(double, double, 1, 16, 1, 1, true),   // 32 x 16
     HJ_K2D(double, double, 1, 8, 1, 1, true),    // 32 x 8
     HJ_K2D(double, double, 1, 16, 4, 1, true),   // 32 x 64

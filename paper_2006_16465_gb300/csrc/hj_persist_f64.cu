@@ -7,6 +7,7 @@
 namespace hj {
 
 static const PersistKernelInfo k_persist[] = {
+    HJ_KP2D(double, double, 1, 8, 4, 1, true),
     HJ_KP2D(double, double, 1, 16, 2, 1, true),
     HJ_KP2D(double, double, 1, 16, 1, 1, true),
     HJ_KP2D(double, double, 1, 8, 1, 1, true),

@@ -6,7 +6,8 @@
 namespace hj {
 
 static const PpcKernelInfo k_ppc[] = {
-    HJ_KPPC(double, double, 1, 16, 2, 1, true, 2),   // 32 x 32
+    HJ_KPPC(double, double, 1, 8, 4, 1, true, 2),   // 32 x 32
+    HJ_KPPC(double, double, 1, 16, 2, 1, true, 2),   // 32 x 32, two warps
     HJ_KPPC(double, double, 1, 16, 1, 1, true, 2),   // 32 x 16
     HJ_KPPC(double, double, 1, 8, 1, 1, true, 2),   // 32 x 8
     HJ_KPPC(double, double, 1, 16, 4, 1, true, 2),   // 32 x 64
