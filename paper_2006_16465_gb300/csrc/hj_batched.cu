@@ -94,6 +94,7 @@ struct PersistLaunch {
     PersistArgs P;
     const void *fn = nullptr;
     int grid = 0, threads = 256, smem = 0;
+    bool late = false;   // persist2d_batch_kernel: cycle c's iterate lies in buffer c % 3
     unsigned char *hb = nullptr, *db = nullptr;
     size_t o_state = 0, o_bar = 0, total = 0;
 };
@@ -121,14 +122,19 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
             tma = make_tmap(&m.mu[0], a.uin, tmap_type(fam, true), ssz, a.ld, cols, rows, ki->bwu, ki->ty + 2) &&
                   make_tmap(&m.mu[1], a.uout, tmap_type(fam, true), ssz, a.ld, cols, rows, ki->bwu, ki->ty + 2) &&
                   make_tmap(&m.mf, a.f, tmap_type(fam, false), tsz, a.ld, cols, rows, ki->bwf, ki->ty);
+            if (tma && probs[p].third)
+                tma = make_tmap(&m.mu[2], probs[p].third, tmap_type(fam, true), ssz, a.ld, cols, rows, ki->bwu, ki->ty + 2);
             if (tma && sig)
                 tma = a.dinv && make_tmap(&m.md, a.dinv, tmap_type(fam, false), tsz, a.ld, cols, rows, ki->bwf, ki->ty);
         }
     }
+    // the kernel of many problems decides one cycle late, over three buffers
+    bool late = tma;
+    for (auto &p : probs) late = late && p.third;
     long long nitems = 0, max_iters = 1;
     for (auto &p : probs) {
         nitems += p.blocks;
-        max_iters = std::max(max_iters, p.a.red.max_cycles + 1);
+        max_iters = std::max(max_iters, p.a.red.max_cycles + (late ? 2 : 1));
     }
     if (nitems > (1LL << 30)) return seterr(HJ_ERR_INVALID_ARG, "too many work items");
     // scratch layout
@@ -142,11 +148,14 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
     const size_t o_part = al(o_ptx + nprob * sizeof(int));
     const size_t o_bar = al(o_part + 2 * nitems * sizeof(double));
     const size_t o_q = al(o_bar + 4 * sizeof(unsigned));          // head, count, changed, (pad)
-    const size_t o_qitems = al(o_q + 4 * sizeof(int) + 2 * sizeof(long long));
+    const size_t o_qitems = al(o_q + 4 * sizeof(int) + 2 * sizeof(long long) + sizeof(int4));   // .. , points, (pad), state
     const size_t o_qoff = al(o_qitems + nitems * sizeof(int));
     const size_t o_ppts = al(o_qoff + nprob * sizeof(int));
     const size_t o_maps = al(o_ppts + nprob * sizeof(long long));
-    const size_t total = al(o_maps + (tma ? nprob * sizeof(PersistMaps) : 0));
+    const size_t o_third = al(o_maps + (tma ? nprob * sizeof(PersistMaps) : 0));
+    const size_t o_qprobs = al(o_third + (late ? nprob * sizeof(void *) : 0));
+    const size_t o_qent = al(o_qprobs + (late ? nprob * sizeof(int) : 0));
+    const size_t total = al(o_qent + (late ? nitems * sizeof(int4) : 0));
     CKS(ensure_scratch(h, total));
     unsigned char *hb = h->h_pstage;
     unsigned char *db = (unsigned char *)h->pscratch;
@@ -169,6 +178,9 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
         }
     }
     if (tma) memcpy(hb + o_maps, maps.data(), nprob * sizeof(PersistMaps));
+    if (late)
+        for (int p = 0; p < nprob; ++p) ((void **)(hb + o_third))[p] = probs[p].third;
+    memset(hb + o_q + 4 * sizeof(int), 0, 2 * sizeof(long long) + sizeof(int4));
     unsigned *hbar = (unsigned *)(hb + o_bar);
     hbar[0] = hbar[1] = 0u;
     ((int *)hbar)[2] = nprob;   // active
@@ -208,6 +220,10 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
     P.q_items = (int *)(db + o_qitems);
     P.q_off = (int *)(db + o_qoff);
     P.prob_points = (const long long *)(db + o_ppts);
+    P.q_state = (int4 *)(db + o_q + 4 * sizeof(int) + 2 * sizeof(long long));
+    P.q_ent = late ? (int4 *)(db + o_qent) : nullptr;
+    P.q_probs = late ? (int *)(db + o_qprobs) : nullptr;
+    P.third = late ? (void *const *)(db + o_third) : nullptr;
     int cap = 0, threads = 256;
     if (classic) {
         int occ = 0;
@@ -218,14 +234,19 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
         threads = ki->threads;
     }
     if (cap < 1) return seterr(HJ_ERR_UNSUPPORTED, "persistent kernel does not fit on an SM");
-    L->grid = (int)std::min<long long>(nitems, cap);
+    // (late: the checks of the cycle before are queue entries too)
+    L->grid = (int)std::min<long long>(nitems + (late ? nprob : 0), cap);
     L->threads = threads;
     L->smem = tma ? ki->tma_smem[sig] : 0;
-    // one problem: one grid barrier per cycle; several: two (reduce, then
-    // retire and rebuild the work queue)
+    // late decisions: one grid barrier per cycle for any number of problems;
+    // else one for a single problem and two for several (reduce, then retire
+    // and rebuild the work queue), which several TMA-staged ones never take
+    if (tma && !late && nprob > 1) return seterr(HJ_ERR_CUDA, "internal: several problems need third iterate buffers");
+    L->late = late;
     L->fn = classic ? (const void *)classic
-            : tma ? (nprob == 1 ? (const void *)ki->tma_one[sig] : (const void *)ki->tma_fn[sig])
-                  : (nprob == 1 ? (const void *)ki->one[sig] : (const void *)ki->fn[sig]);
+            : late ? (const void *)ki->tma_fn[sig]
+            : tma ? (const void *)ki->tma_one[sig]
+            : nprob == 1 ? (const void *)ki->one[sig] : (const void *)ki->fn[sig];
     L->hb = hb;
     L->db = db;
     L->o_state = o_state;
@@ -269,7 +290,8 @@ namespace bsched {
 // ---------------------------------------------------------------------------
 // Device side of the refinement loop over a batch.  Every problem has binary64
 // iterate buffers u[0] (the caller's) and u[1], a binary32 residual r32 (the
-// inner right-hand side), two correction buffers d[0], d[1] and an outer state.
+// inner right-hand side), correction buffers d[0], d[1], d[2] (the plain-staging
+// engine uses two of them) and an outer state.
 // One refinement step is, for the problems still refining:
 //   zero d[0]; inner cycles A d = r32 (the persistent launch, d[0] -> d[1] ...);
 //   u[cur ^ 1] = u[cur] + d, r = f - A u[cur ^ 1] (binary64), ||r||;
@@ -281,7 +303,7 @@ struct BDev {
     const double *f;
     double *u[2];
     float *r32;
-    void *d[2];
+    void *d[3];
     const double *sigma;
     long long ld, ld_in;      // pitch of f, u, sigma; pitch of r32 and d
     int nx, ny;
@@ -308,6 +330,7 @@ struct BatchArgs {
     double *aux_part;         // per aux item: its share of ||r||^2
     int *count;               // problems still refining (read by the host)
     int nprob, naux;
+    int nbuf;                 // correction buffers the inner cycles rotate through
     double tol;
     DbgWord *dbg;             // debug builds: the index-check word
 };
@@ -361,7 +384,7 @@ __global__ void __launch_bounds__(256) batch_residual_kernel(const BatchArgs A) 
             const double *u = b.u[o.cur];
             double uc = u[q], uW = u[q - 1], uE = u[q + 1], uS = u[q - b.ld], uN = u[q + b.ld];
             if constexpr (!INIT) {
-                const DS *d = (const DS *)b.d[A.state[p].done & 1];
+                const DS *d = (const DS *)b.d[A.state[p].done % A.nbuf];
                 uc = __dadd_rn(uc, corr(d + q2));
                 uW = __dadd_rn(uW, corr(d + q2 - 1));
                 uE = __dadd_rn(uE, corr(d + q2 + 1));
@@ -452,7 +475,7 @@ struct BProb {
     double *u;               // caller's iterate
     double *u2;              // second binary64 buffer
     float *r32;              // binary32 residual (inner RHS)
-    void *dA, *dB;           // correction buffers
+    void *dA, *dB, *dC;      // correction buffers
     float *dinv;             // per-point 1/d in binary32 (some problem of the batch has sigma)
 };
 
@@ -558,7 +581,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         b.u = (double *)u[i];
         arena += ((size_t)b.rows * b.d.ld * 8 + 255) / 256 * 256;    // u2
         arena += (b.nin * 4 + 255) / 256 * 256;                       // r32
-        arena += 2 * ((b.nin * dsz + 255) / 256 * 256);               // dA, dB
+        arena += 3 * ((b.nin * dsz + 255) / 256 * 256);               // dA, dB, dC
         if (sig_any) arena += (b.nin * 4 + 255) / 256 * 256;          // per-point 1/d (binary32)
     }
     if (arena > h->barena_bytes) {
@@ -578,6 +601,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         b.r32 = (float *)ap; ap += (b.nin * 4 + 255) / 256 * 256;
         b.dA = ap; ap += (b.nin * dsz + 255) / 256 * 256;
         b.dB = ap; ap += (b.nin * dsz + 255) / 256 * 256;
+        b.dC = ap; ap += (b.nin * dsz + 255) / 256 * 256;
         b.dinv = nullptr;
         if (sig_any) {
             b.dinv = (float *)ap; ap += (b.nin * 4 + 255) / 256 * 256;
@@ -589,6 +613,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         CKR(cudaMemsetAsync(b.r32, 0, b.nin * 4, s));
         CKR(cudaMemsetAsync(b.dA, 0, b.nin * dsz, s));
         CKR(cudaMemsetAsync(b.dB, 0, b.nin * dsz, s));
+        CKR(cudaMemsetAsync(b.dC, 0, b.nin * dsz, s));
     }
     // the inner engine over every problem of the batch (its work queue holds
     // the items of the problems still refining)
@@ -602,6 +627,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         q.a.f = b.r32;
         q.a.uin = b.dA;
         q.a.uout = b.dB;
+        q.third = b.dC;
         q.a.dinv = b.dinv;
         q.a.red.tol = par.inner_tol;
         q.a.red.tol2 = par.inner_tol * par.inner_tol * (1.0 + 1e-9);
@@ -630,6 +656,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         x.r32 = b.r32;
         x.d[0] = b.dA;
         x.d[1] = b.dB;
+        x.d[2] = b.dC;
         x.sigma = b.d.sigma;
         x.ld = b.d.ld;
         x.ld_in = b.ld_in;
@@ -689,6 +716,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
     B.count = (int *)(dm + m_word);
     B.nprob = nprob;
     B.naux = (int)naux;
+    B.nbuf = L.late ? 3 : 2;
     B.tol = par.tol;
     B.dbg = debug_word();
     const dim3 bg = batch_grid((int)naux, h->nsm), bb(32, 8);

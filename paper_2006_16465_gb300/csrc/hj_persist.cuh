@@ -18,6 +18,8 @@
 //   barrier  (grid-wide, bounded): the last CTA to arrive rebuilds the queue
 //            if a problem retired, resets its head and logs the cycle's end
 //            time; stop when no problem is active.
+// The TMA-staged kernel of many problems (hj_persist_tma.cuh) needs one barrier
+// per cycle instead: it decides a cycle later, over three iterate buffers.
 // Problems of different sizes, stencils, k and tolerances share the launch.
 // Single-problem launches keep a static stride over the problem's items.
 // Every barrier wait is bounded by wall time (%globaltimer); on expiry the
@@ -67,6 +69,11 @@ struct PersistArgs {
     int *q_off;              // [nprob] scratch of the rebuild: first entry of each problem, -1 if retired
     const long long *prob_points;   // per problem: interior points
     long long *q_points;     // interior points of the active problems
+    // work queue of the TMA-staged multi-problem kernel (persist2d_batch_kernel)
+    int4 *q_ent;             // [nitems] {item, problem, block x, block y} of the active problems
+    int *q_probs;            // [nprob] the active problems
+    int4 *q_state;           // {entries in q_ent, active problems, CTAs of the next cycle, number of rebuilds}
+    void *const *third;      // per problem: the third iterate buffer
     // per-cycle log (nullable): [2 * n] = end time (ns), [2 * n + 1] = active points of the next cycle
     unsigned long long *tlog;
     long long *tlog_n;

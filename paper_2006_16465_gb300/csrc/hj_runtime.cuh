@@ -151,6 +151,7 @@ struct PersistProblem {
                       // red.tol, red.max_cycles, red.scale (red.hist for a single problem)
     int blocks_x;     // CTAs along x (2D tiles, or 1D groups of tiles)
     int blocks;       // CTAs in total
+    void *third = nullptr;   // third iterate buffer (many problems, TMA staging: decisions one cycle late)
 };
 // classic: run the grid-sync classic kernel (one problem, blocks of points as items)
 // fam >= 0 (the kernels' family) lets 2D problems stage by TMA (pipeline != 0).
