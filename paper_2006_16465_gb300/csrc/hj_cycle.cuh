@@ -109,6 +109,61 @@ __device__ __forceinline__ T point_update(const Coef<T> &k, T g, T iv, T W, T E,
     }
 }
 
+// Correctly rounded product of a binary64 value and a constant on the integer
+// pipes: the 53-bit significand of x times the constant's (as 64 bits, top bit
+// set) as four 32 x 32 -> 64 multiplications, then one normalising shift and
+// round-to-nearest-even on the 64 bits below the kept 53.  Some 30 instructions
+// against the 64 to 77 clocks that the FP64 pipe takes for its one, and they
+// run beside it: of the six operations a point has left (update_from_products),
+// the four sums keep the FP64 pipe and the two products leave it.  Measured with
+// 32 x 32 subdomains on four warps, us a cycle: 3001 x 2003, k = 16 1315 -> 836,
+// k = 4 347 -> 230, k = 1 104 -> 78; 900 x 800, k = 16 178 -> 137 (eight warps
+// 175 -> 123); 256 x 256 (one subdomain per SM, bound by latency) unchanged.
+// Exact as long as x and the product are normal numbers well inside the range:
+// `bad` collects the largest exponent-field distance from the constant's lower
+// limit, and the caller repeats the work on the FP64 pipe where it exceeds
+// `span` (zeros, subnormals, infinities, NaN, and products near the limits).
+struct MulConst {
+    unsigned ch, cl;      // significand of the constant, 64 bits
+    unsigned k;           // exponent term of the result's high word
+    unsigned sgn;
+    unsigned emin, span;  // exponent fields of x (in place, bits 20..30) that are handled: [emin, emin + span]
+};
+__device__ __forceinline__ MulConst make_mul_const(double c) {
+    MulConst m;
+    const unsigned hi = (unsigned)__double2hiint(c), lo = (unsigned)__double2loint(c);
+    const int ec = (int)((hi >> 20) & 0x7ffu);
+    m.ch = 0x80000000u | (hi << 11) | (lo >> 21);
+    m.cl = lo << 11;
+    m.sgn = hi & 0x80000000u;
+    m.k = (unsigned)(ec - 1024) << 20;
+    // x's exponent field e >= 1, and the product's, e + ec - 1022 or one less, within [1, 2045]
+    const int e0 = ec > 1024 ? 1 : 1025 - ec, e1 = ec < 1021 ? 2046 : 3067 - ec;
+    const bool ok = ec >= 1 && ec <= 2046 && e0 <= 2046 && e1 >= e0;
+    m.emin = ok ? (unsigned)e0 << 20 : 1u;   // (a field in place is never 1: nothing is handled)
+    m.span = ok ? (unsigned)(e1 - e0) << 20 : 0u;
+    return m;
+}
+__device__ __forceinline__ double mul_const(double x, const MulConst &m, unsigned &bad) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned e = hi & 0x7ff00000u, xm = (hi & 0x000fffffu) | 0x00100000u;
+    const unsigned long long p00 = (unsigned long long)lo * m.cl;
+    const unsigned long long p01 = (unsigned long long)lo * m.ch + (unsigned)(p00 >> 32);
+    const unsigned long long p10 = (unsigned long long)xm * m.cl + (unsigned)p01;
+    const unsigned long long p11 = (unsigned long long)xm * m.ch + (unsigned)(p01 >> 32) + (unsigned)(p10 >> 32);
+    // the product's bits 64.. (w3:w2, in [2^51, 2^53)) and the 32 below with a sticky bit
+    unsigned w3 = (unsigned)(p11 >> 32), w2 = (unsigned)p11, w1 = (unsigned)p10 | ((unsigned)p00 != 0u ? 1u : 0u);
+    const unsigned s = w3 & 0x00100000u, sh = (s >> 20) ^ 1u;   // bit 52 set: no shift
+    w3 = __funnelshift_l(w2, w3, sh);
+    w2 = __funnelshift_l(w1, w2, sh);
+    w1 <<= sh;
+    const unsigned long long r = (unsigned long long)w1 + (0x7fffffffu + (w2 & 1u));   // carry: round up
+    const unsigned long long v = (((unsigned long long)w3 << 32) | w2) + (unsigned)(r >> 32);
+    bad = max(bad, e - m.emin);
+    const unsigned oh = ((unsigned)(v >> 32) + e + s + m.k) ^ ((hi ^ m.sgn) & 0x80000000u);
+    return __hiloint2double((int)oh, (int)(unsigned)v);
+}
+
 // Binary64 update from the rounded products c_X u_X of the four neighbours (two
 // in 1D): the sums and the final scaling of point_update, in its order.
 //
@@ -121,11 +176,13 @@ __device__ __forceinline__ T point_update(const Coef<T> &k, T g, T iv, T W, T E,
 // term of p's right neighbour and the E term of its left one, bit for bit:
 // formed once by its owner, it replaces one of the two multiplications, and
 // with all four equal three of the four.  9 operations a point become 7 or 6
-// (1D: 5 become 4), with every rounding where it was.  Measured: 10 cycles of
-// k = 16 on 3001 x 2003 (7 operations) 17.9 -> 14.5 ms, a 256 x 256 solve to
-// 1e-6 (6 operations) 0.77 -> 0.59 s, a 512-point line to 1e-6 0.371 -> 0.351 s.
+// (1D: 5 become 4), with every rounding where it was.  Measured by itself, on two
+// warps per subdomain: 10 cycles of k = 16 on 3001 x 2003 (7 operations) 17.9 ->
+// 14.5 ms, a 256 x 256 solve to 1e-6 (6 operations) 0.77 -> 0.59 s, a 512-point
+// line to 1e-6 0.371 -> 0.351 s.
 template <typename T, bool SIG, bool D2, bool WANT_RES>
-__device__ __forceinline__ T update_from_products(const Coef<T> &k, T g, T iv, T pW, T pE, T pS, T pN, T old, T &res) {
+__device__ __forceinline__ T update_from_products(const Coef<T> &k, T g, T iv, T pW, T pE, T pS, T pN, T old, T &res,
+                                                  const MulConst *mi = nullptr, unsigned *bad = nullptr) {
     double acc = __dadd_rn(pW, pE);
     if constexpr (D2) {
         acc = __dadd_rn(acc, pS);
@@ -136,6 +193,7 @@ __device__ __forceinline__ T update_from_products(const Coef<T> &k, T g, T iv, T
         const double dp = SIG ? __drcp_rn(iv) : (double)k.dconst;
         res = (T)__dsub_rn(t, __dmul_rn(dp, old));
     }
+    if (mi) return (T)mul_const(t, *mi, *bad);   // (known at compile time)
     return (T)__dmul_rn(t, SIG ? (double)iv : (double)k.invd);
 }
 
@@ -531,6 +589,10 @@ sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, 
     const unsigned m_top = lane_mask(hb > 0), m_bot = lane_mask(hb < H - 1);         // bands with a band above / below
     typedef typename std::conditional<EXACT, double, T>::type Acc;
     Acc acc = 0;
+    // Products on the integer pipes (INT) where a band's saved values fit in
+    // registers beside it; both directions' products are formed there, so the
+    // case of four equal coefficients needs no variant of its own.
+    constexpr bool INTOK = EXACT && R * C <= 8;
     // SYM: which neighbour products are shared (shared_products; binary64 only).
     // With sharing, t.hx, t.top and t.bot hold products (c times the halo or
     // neighbouring row), t.v holds values.
@@ -538,10 +600,34 @@ sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, 
     constexpr int SYM = decltype(sym_tag)::value;
     auto px = [&](T x) -> T { if constexpr (SYM != 0) return (T)__dmul_rn(kc.cW, x); else return x; };   // W/E term
     auto py = [&](T x) -> T { if constexpr (SYM != 0) return (T)__dmul_rn(kc.cS, x); else return x; };   // S/N term
+    // the same on the integer pipes (INT); bx, by, bi collect what they cannot do
+    MulConst mx, my, mi;
+    unsigned bx = 0, by = 0, bi = 0;
+    if constexpr (SYM != 0 && INTOK) {
+        mx = make_mul_const(kc.cW);
+        my = make_mul_const(kc.cS);
+        if constexpr (!SIG) mi = make_mul_const(kc.invd);
+    }
+    bool fast = SYM != 0 && INTOK;   // cleared once a subiteration met values the integer product leaves out
+    auto failed = [&]() -> bool {
+        bool f = bx > mx.span || by > my.span;
+        if constexpr (!SIG) f = f || bi > mi.span;
+        bx = by = bi = 0;
+        return __any_sync(FULL, f);
+    };
     // products of the band's first and last row (formed with the exchange)
     T e0[SYM ? C : 1], eR[SYM ? C : 1];
     auto edge_products = [&]() {
         if constexpr (SYM != 0) {
+            if (INTOK && fast) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    e0[c] = mul_const(t.v[0][c], my, by);
+                    eR[c] = mul_const(t.v[R - 1][c], my, by);
+                }
+                if (!failed()) return;
+                fast = false;
+            }
 #pragma unroll
             for (int c = 0; c < C; ++c) {
                 e0[c] = py(t.v[0][c]);
@@ -560,8 +646,11 @@ sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, 
         }
         edge_products();
     }
-    auto sweep = [&](auto first_tag) {
+    auto sweep_as = [&](auto first_tag, auto int_tag) {
         constexpr bool FIRST = decltype(first_tag)::value;
+        constexpr bool INT = decltype(int_tag)::value;
+        auto tx = [&](T x) -> T { if constexpr (INT) return mul_const(x, mx, bx); else return px(x); };
+        auto ty = [&](T x) -> T { if constexpr (INT) return mul_const(x, my, by); else return py(x); };
         T prev[C];                   // S terms of the row: the old row below (SYM: its products)
         T mid[SYM ? C : 1];          // SYM: S/N products of the row itself
 #pragma unroll
@@ -579,8 +668,8 @@ sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, 
                     hor[c] = cur[c];
                     nxt[c] = (r == R - 1) ? t.bot[c] : t.v[r < R - 1 ? r + 1 : 0][c];
                 } else {
-                    hor[c] = SYM == 2 ? mid[c] : px(cur[c]);
-                    nxt[c] = (r == R - 1) ? t.bot[c] : (r == R - 2) ? eR[c] : py(t.v[r < R - 1 ? r + 1 : 0][c]);
+                    hor[c] = SYM == 2 ? mid[c] : tx(cur[c]);
+                    nxt[c] = (r == R - 1) ? t.bot[c] : (r == R - 2) ? eR[c] : ty(t.v[r < R - 1 ? r + 1 : 0][c]);
                 }
             }
             const T left = mask_sel(m_first, t.hx[r], __shfl_up_sync(FULL, hor[C - 1], 1));
@@ -596,7 +685,7 @@ sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, 
                                                                          res);
                 else
                     nv = update_from_products<T, SIG, true, FIRST && RES>(kc, t.g[r][c], dvc, W, E, prev[c], nxt[c],
-                                                                          cur[c], res);
+                                                                          cur[c], res, INT && !SIG ? &mi : nullptr, &bi);
                 if constexpr (PART) {
                     const bool act = (yb + r <= ny) && (xl + c <= nx);
                     nv = act ? nv : cur[c];
@@ -619,6 +708,29 @@ sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, 
                 }
             }
         }
+    };
+    // one subiteration: the products on the integer pipes, repeated without them
+    // from the saved values where they do not cover what it met (the residual's
+    // subiteration has FP64 work of its own and a body of its own: left as is)
+    auto sweep = [&](auto first_tag) {
+        constexpr bool FIRST = decltype(first_tag)::value && RES;
+        if constexpr (SYM != 0 && INTOK && !FIRST) {
+            if (fast) {
+                T old[R][C];
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int c = 0; c < C; ++c) old[r][c] = t.v[r][c];
+                sweep_as(std::integral_constant<bool, false>(), std::integral_constant<bool, true>());
+                if (!failed()) return;
+                fast = false;
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int c = 0; c < C; ++c) t.v[r][c] = old[r][c];
+            }
+        }
+        sweep_as(std::integral_constant<bool, FIRST>(), std::integral_constant<bool, false>());
     };
     int par = 0;
     // before each subiteration after the first: the rows next to each band
@@ -694,8 +806,13 @@ sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, 
     };
     if constexpr (EXACT) {
         const int sym = shared_products(kc);   // the same for every thread
-        if (sym == 2) run(std::integral_constant<int, 2>());
-        else if (sym == 1) run(std::integral_constant<int, 1>());
+        if constexpr (!INTOK) {
+            if (sym == 2) {
+                run(std::integral_constant<int, 2>());
+                return acc;
+            }
+        }
+        if (sym >= 1) run(std::integral_constant<int, 1>());
         else run(std::integral_constant<int, 0>());
     } else {
         run(std::integral_constant<int, 0>());

@@ -64,3 +64,21 @@ def test_multigrid_modes(shape, tile):
     for _ in range(2):
         ref = oracle.mg_vcycle(p.st, p.f, ref, L, 1, 1, tile[0], tile[1], 3, 0.8)
     assert np.array_equal(got, ref), rel_max(got, ref)
+
+
+@pytest.mark.parametrize("scale,zeros", [(1e-303, False), (1e-306, True), (1e-311, False), (1e295, True), (1.0, True)])
+@pytest.mark.parametrize("shape,asym", [((64, 64), False), ((71, 38), False)])
+def test_products_at_the_edges_of_the_range(shape, asym, scale, zeros):
+    """Products formed on the integer pipes cover normal numbers; zeros, subnormal
+    values and products near the limits take the FP64 pipe, per subiteration."""
+    import paper_2006_16465_gb300 as hj
+    p = W.random_bc_problem(2, *shape, seed=77, sigma_kind="none", asym=asym)
+    p.f *= scale
+    p.u0 *= scale
+    if zeros:   # half the grid exactly zero, its front moving one row a subiteration
+        p.f[: shape[1] // 2] = 0.0
+        p.u0[: shape[1] // 2] = 0.0
+    for tx, ty, th in hj.hj_tile_variants(2, hj.PRECISIONS["f64"]):
+        got = _cycles(p, 2, tile_x=tx, tile_y=ty, tile_threads=th, k=5, fixed_cycles=3, pipeline=0)
+        ref = oracle.run_fixed(p.st, p.f, p.u0, 3, tx, ty, 5)
+        assert np.array_equal(got, ref), (tx, ty, th, rel_max(got, ref))
