@@ -332,6 +332,13 @@ int get_graph(hj_handle *h, void (*fn)(Args), dim3 grid, dim3 block, int smem, c
     return HJ_OK;
 }
 
+// Whether the per-point-coefficient cycles run the kernel with four rows a warp
+// (vc2d_rows_kernel: binary32 2D subdomains 32 wide, 4 to 32 rows high).
+bool vc_rows(const hj_handle *h) {
+    return h->d.coef && h->d.dim == 2 && h->fam_outer == FAM_F32 && h->p.tile_x == 32 && h->p.tile_y % 4 == 0 &&
+           h->p.tile_y <= 32;
+}
+
 // Launch plan for one iteration kernel: either the one-CTA-per-tile kernel
 // (CycArgs) or the TMA-pipelined kernel (PpcArgs) with its two argument blocks.
 // Converging runs of the pipelined kernel rotate three iterate buffers and
@@ -560,6 +567,12 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
         pl->grid = h->d.dim == 2 ? dim3((nx + tx - 1) / tx, (ny + ty - 1) / ty) : dim3((nx + tx - 1) / tx, ny);
         pl->block = h->d.dim == 2 ? dim3(tx, ty) : dim3(tx);
         pl->smem = 2 * (tx + 2) * (h->d.dim == 2 ? ty + 2 : 1) * (fam == FAM_F64 ? 8 : 4);
+        if (vc_rows(h)) {
+            // binary32, 32 columns wide: four rows a warp, the same subdomains
+            pl->fn = vk->rows[res];
+            pl->block = dim3(32 * (ty / 4));
+            pl->smem = 0;
+        }
         if (classic) pl->a[0].k = pl->a[1].k = 1;
         pl->ppc = false;
         return HJ_OK;
@@ -1063,7 +1076,8 @@ void fill_stats_config(const hj_handle *h, hj_stats *st, double t0) {
     st->tile_y = h->d.dim == 2 ? h->p.tile_y : 1;
     st->k = h->p.k;
     const TileKernelInfo *tk = h->ir ? h->k_inner : h->k_outer;
-    st->tile_threads = tk ? tk->threads / tk->tiles_per_cta
+    st->tile_threads = tk            ? tk->threads / tk->tiles_per_cta
+                       : vc_rows(h) ? 8 * h->p.tile_y
                           : (h->d.coef || h->p.method == HJ_METHOD_MG) ? h->p.tile_x * (h->d.dim == 2 ? h->p.tile_y : 1)
                           : h->k3                                      ? 32
                                                                        : 0;

@@ -37,7 +37,7 @@ const TileKernelInfo *tile_kernels_f64(int *n) {
 }
 const TileKernelInfo *classic_kernels_f64(int *n) { *n = 2; return k_classic; }
 
-static const VcKernelInfo k_vc = HJ_KVC(double, double, true);
+static const VcKernelInfo k_vc = HJ_KVC(double, double, true, nullptr, nullptr);
 const VcKernelInfo *vc_kernels_f64() { return &k_vc; }
 
 }  // namespace hj

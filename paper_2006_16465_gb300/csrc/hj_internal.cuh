@@ -444,8 +444,11 @@ struct TileKernelInfo {
 
 // Variable-coefficient kernels: [dim - 1][res], one thread per point, dynamic
 // shared memory 2 * (tile_x + 2) * (tile_y + 2) elements of the compute type.
+// rows[res]: 2D subdomains 32 wide and 4, 8, .. 32 high (tile_y / 4 warps; null
+// where not built).
 struct VcKernelInfo {
     CycKernel fn[2][2];
+    CycKernel rows[2];
 };
 const VcKernelInfo *vc_kernels_f64();
 const VcKernelInfo *vc_kernels_f32();
