@@ -489,14 +489,15 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
             const int smem = t3->ppc_smem;
             CKR(ensure_dyn_smem(h->dev, (const void *)fn, smem));
             int occ = 0;
-            CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 32, smem));
+            CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 32 * t3->ppc_ns, smem));
             if (occ < 1) return seterr(HJ_ERR_UNSUPPORTED, "3D pipelined kernel does not fit on an SM");
             if (h->p.ctas_per_sm > 0) occ = std::min(occ, h->p.ctas_per_sm);
             else if (t3->ppc_cps > 0) occ = std::min(occ, t3->ppc_cps);
-            const int tiles_x = (nx + t3->tx - 1) / t3->tx, tiles_y = (ny + t3->ty - 1) / t3->ty;
+            const int cx = t3->tx * t3->ppc_ns;   // columns a CTA takes at a time
+            const int tiles_x = (nx + cx - 1) / cx, tiles_y = (ny + t3->ty - 1) / t3->ty;
             const int ntiles = tiles_x * tiles_y * ((h->d.nz + t3->tz - 1) / t3->tz);
             const int grid = std::min(ntiles, occ * h->nsm);
-            const int bw = (t3->tx + 2 + 3) / 4 * 4;   // box width: the kernel's BX
+            const int bw = (cx + 2 + 3) / 4 * 4;   // box width: the kernel's BX
             void *bufs[3] = {b0, b1, b2};
             pl->deferred = res;
             pl->period = res ? kPpcPeriod : 2;
@@ -525,7 +526,7 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
             pl->pfn = fn;
             pl->smem = smem;
             pl->grid = dim3(grid);
-            pl->block = dim3(32);
+            pl->block = dim3(32 * t3->ppc_ns);
             return HJ_OK;
         }
         if (classic) {

@@ -547,10 +547,16 @@ __global__ void __launch_bounds__(32 * NW, 3) hier3d_pk_kernel(const CycArgs a) 
 // Every wait on the mbarrier is bounded; on expiry the kernel records the
 // error, waits (bounded) for its copy in flight and returns.
 // ---------------------------------------------------------------------------
-template <int LX, int RY, int RZ>
+// NS: subdomains side by side along x in one CTA, a warp each, sharing one pair
+// of boxes: 16-wide subdomains in pairs turn 80-byte box rows into 144-byte ones,
+// which the copy engine and DRAM serve better, and copy the halo columns between
+// the two once.  Measured at 512^3, k = 4, us a cycle: 16 x 8 x 8
+// 328 -> 311 (k = 1 320 -> 276), 16 x 8 x 4 334 -> 327; at full residency, where
+// single subdomains had to be held to 8 and 12 CTAs per SM.
+template <int LX, int RY, int RZ, int NS>
 struct Ppc3Layout {
     static constexpr int LY = 32 / LX, TX = 2 * LX, TY = LY * RY, TZ = RZ;
-    static constexpr int BX = round_up(TX + 2, 4);   // box width (iterate and RHS), 16-byte multiple
+    static constexpr int BX = round_up(NS * TX + 2, 4);   // box width (iterate and RHS), 16-byte multiple
     static constexpr int UB = BX * (TY + 2) * (TZ + 2) * 4, FB = BX * TY * TZ * 4;
     static constexpr int UB_AL = round_up(UB, 128), FB_AL = round_up(FB, 128);
     static constexpr int TX_BYTES = UB + FB;
@@ -558,9 +564,9 @@ struct Ppc3Layout {
     static constexpr int SMEM = BAR_OFF + 8 + 128;   // + room to align the base to 128 bytes
 };
 
-template <int LX, int RY, int RZ, bool RES>
-__global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcArgs P) {
-    using L = Ppc3Layout<LX, RY, RZ>;
+template <int LX, int RY, int RZ, int NS, bool RES>
+__global__ void __launch_bounds__(32 * NS) ppc3d_kernel(const __grid_constant__ PpcArgs P) {
+    using L = Ppc3Layout<LX, RY, RZ, NS>;
     using P3 = Pk3<LX, RY, RZ>;
     constexpr int LY = L::LY, TX = L::TX, TY = L::TY, TZ = L::TZ, BX = L::BX;
     static_assert(LY > 1, "the first and last lane groups are different groups");
@@ -568,9 +574,11 @@ __global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcAr
     const bool reducer = blockIdx.x == gridDim.x - 1;
     if constexpr (RES) {
         volatile Ctl *ctl = a.red.ctl;
-        if (ctl->done >= 0) return;
+        // one answer for the whole CTA: the reducer of this launch may be setting done now
+        const int done = ctl->done >= 0;
+        if (NS == 1 ? __any_sync(0xffffffffu, done) : __syncthreads_or(done)) return;
         if (ctl->fold_only[P.parity]) {
-            if (reducer) deferred_fold<1>(P);
+            if (reducer) deferred_fold<NS>(P);
             return;
         }
     }
@@ -578,7 +586,7 @@ __global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcAr
     unsigned char *smem = smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u);
     float *su = (float *)smem, *sf = (float *)(smem + L::UB_AL);
     uint64_t *bar = (uint64_t *)(smem + L::BAR_OFF);
-    const int lane = threadIdx.x;
+    const int lane = threadIdx.x & 31, ws = threadIdx.x >> 5, tid = threadIdx.x;   // ws: this warp's subdomain of the CTA's NS
     const int lx = lane % LX, gy = lane / LX;
     const bool wl = lx == 0, el = lx == LX - 1, sl = gy == 0, nl = gy == LY - 1;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
@@ -587,19 +595,19 @@ __global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcAr
     auto issue = [&](int tile) {
         const int bx = tile % txs, by = (tile / txs) % tys, bz = tile / (txs * tys);
         mbar_expect_tx(bar, L::TX_BYTES);
-        tma_load_3d(su, &P.mu, bar, bx * TX, by * TY, bz * TZ);
-        tma_load_3d(sf, &P.mf, bar, bx * TX, by * TY + 1, bz * TZ + 1);
+        tma_load_3d(su, &P.mu, bar, bx * NS * TX, by * TY, bz * TZ);
+        tma_load_3d(sf, &P.mf, bar, bx * NS * TX, by * TY + 1, bz * TZ + 1);
     };
-    if (lane == 0) {
+    if (tid == 0) {
         mbar_init(bar, 1);
         fence_mbar_init();
     }
     __syncthreads();
-    if (lane == 0 && mine > 0) issue(blockIdx.x);
+    if (tid == 0 && mine > 0) issue(blockIdx.x);
     // the last CTA has the fewest subdomains when the grid does not divide
     // them: it folds the previous launch's residual while its first copy lands
     if constexpr (RES) {
-        if (reducer) deferred_fold<1>(P);
+        if (reducer) deferred_fold<NS>(P);
     }
     const Coef3<float> kc = make_coef3<float>(a);
     const long long ld = a.ld, ps = a.ps;
@@ -615,16 +623,16 @@ __global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcAr
         if (__syncthreads_or(!ok)) { failed = true; break; }
         const int tile = blockIdx.x + i * gridDim.x;
         const int bx = tile % txs, by = (tile / txs) % tys, bz = tile / (txs * tys);
-        const int x0 = 1 + bx * TX, y0 = 1 + by * TY, z0 = 1 + bz * TZ;
+        const int x0 = 1 + (bx * NS + ws) * TX, y0 = 1 + by * TY, z0 = 1 + bz * TZ;
         const int x = x0 + 2 * lx, yl = y0 + gy * RY;
         const bool full = x0 + TX - 1 <= nx && y0 + TY - 1 <= ny && z0 + TZ - 1 <= nz;
         // stage from the boxes: iterate box element (X, Y, Z) relative to
         // (x0 - 1, y0 - 1, z0 - 1), RHS box element relative to (x0 - 1, y0, z0)
         P3 t;
         {
-            const int cx = 1 + 2 * lx, ry = gy * RY;
+            const int cx = 1 + ws * TX + 2 * lx, ry = gy * RY;
             auto U = [&](int X, int Y, int Z) -> float { return su[(Z * (TY + 2) + Y) * BX + X]; };
-            const int xo = wl ? 0 : cx + 2, yo = sl ? 0 : ry + RY + 1;
+            const int xo = wl ? ws * TX : cx + 2, yo = sl ? 0 : ry + RY + 1;
 #pragma unroll
             for (int z = 0; z < RZ; ++z) {
 #pragma unroll
@@ -650,10 +658,11 @@ __global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcAr
             }
         }
         __syncthreads();   // every lane is done with the boxes
-        if (lane == 0 && i + 1 < mine) {
+        if (tid == 0 && i + 1 < mine) {
             fence_proxy_async_smem();
             issue(blockIdx.x + (i + 1) * gridDim.x);
         }
+        if (NS > 1 && x0 > nx) continue;   // beyond the grid's edge (warp-uniform; no barrier below)
         pk3_fold<LX, RY, RZ>(t, kc, wl, el, sl, nl);
         if (full) acc += pk3_sweeps<LX, RY, RZ, RES, false>(t, kc, a.k, wl, el, sl, nl, x, yl, z0, nx, ny, nz);
         else acc += pk3_sweeps<LX, RY, RZ, RES, true>(t, kc, a.k, wl, el, sl, nl, x, yl, z0, nx, ny, nz);
@@ -661,7 +670,7 @@ __global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcAr
     }
     if (failed) {
         // record the expiry, wait (bounded) for the copy in flight, return
-        if (lane == 0) {
+        if (tid == 0) {
             atomicExch(a.err, HJ_ERR_TIMEOUT);
             long long spins = 0;
             while (!mbar_try_wait(bar, (unsigned)i & 1u) && ++spins <= P.spin_limit) {
@@ -670,7 +679,7 @@ __global__ void __launch_bounds__(32) ppc3d_kernel(const __grid_constant__ PpcAr
         __syncthreads();
         return;
     }
-    if constexpr (RES) write_cta_partial<1>(P.part_w + blockIdx.x, acc);
+    if constexpr (RES) write_cta_partial<NS>(P.part_w + blockIdx.x, acc);
 }
 
 // ---------------------------------------------------------------------------
@@ -911,21 +920,21 @@ __global__ void __launch_bounds__(256) classic3d_kernel(const CycArgs a) {
      {hj::hier3d_kernel<S, T, LX, RY, RZ, NW, EX, false>, hj::hier3d_kernel<S, T, LX, RY, RZ, NW, EX, true>}, \
      {hj::hier3d_pf_kernel<S, T, LX, RY, RZ, NW, EX, false>,                                         \
       hj::hier3d_pf_kernel<S, T, LX, RY, RZ, NW, EX, true>},                                         \
-     (int)((NW) * hj::Pf3Layout<T, LX, RY, RZ>::PER_WARP * sizeof(T)), {nullptr, nullptr}, 0, 0}
+     (int)((NW) * hj::Pf3Layout<T, LX, RY, RZ>::PER_WARP * sizeof(T)), {nullptr, nullptr}, 0, 0, 1}
 
 // binary32 entry of the same TX x TY x TZ shape: the two-column kernel, whose
 // LX / 2 lanes span x with RY / 2 rows per lane group, the one-column
 // prefetching kernel, and the TMA-pipelined two-column kernel with its
-// resident CTAs per SM (CPS, measured per shape: more copies in flight slowed
+// subdomains per CTA (NS) and its resident CTAs per SM (CPS, measured per shape: more copies in flight slowed
 // the 16-wide boxes sharply)
-#define HJ_K3D_F32(LX, RY, RZ, NW, CPS)                                                              \
+#define HJ_K3D_F32(LX, RY, RZ, NW, NS, CPS)                                                              \
     {(LX), (32 / (LX)) * (RY), (RZ), 32 * (NW), (NW),                                               \
      {hj::hier3d_pk_kernel<(LX) / 2, (RY) / 2, RZ, NW, false>, hj::hier3d_pk_kernel<(LX) / 2, (RY) / 2, RZ, NW, true>}, \
      {hj::hier3d_pf_kernel<float, float, LX, RY, RZ, NW, false, false>,                              \
       hj::hier3d_pf_kernel<float, float, LX, RY, RZ, NW, false, true>},                              \
      (int)((NW) * hj::Pf3Layout<float, LX, RY, RZ>::PER_WARP * sizeof(float)),                       \
-     {hj::ppc3d_kernel<(LX) / 2, (RY) / 2, RZ, false>, hj::ppc3d_kernel<(LX) / 2, (RY) / 2, RZ, true>},  \
-     hj::Ppc3Layout<(LX) / 2, (RY) / 2, RZ>::SMEM, (CPS)}
+     {hj::ppc3d_kernel<(LX) / 2, (RY) / 2, RZ, NS, false>, hj::ppc3d_kernel<(LX) / 2, (RY) / 2, RZ, NS, true>}, \
+     hj::Ppc3Layout<(LX) / 2, (RY) / 2, RZ, NS>::SMEM, (CPS), (NS)}
 
 // the same without the pipelined kernel (8-wide boxes: 48-byte rows, which
 // the copy engine moves too slowly to gain on the one-warp kernel)
@@ -934,4 +943,4 @@ __global__ void __launch_bounds__(256) classic3d_kernel(const CycArgs a) {
      {hj::hier3d_pk_kernel<(LX) / 2, (RY) / 2, RZ, NW, false>, hj::hier3d_pk_kernel<(LX) / 2, (RY) / 2, RZ, NW, true>}, \
      {hj::hier3d_pf_kernel<float, float, LX, RY, RZ, NW, false, false>,                              \
       hj::hier3d_pf_kernel<float, float, LX, RY, RZ, NW, false, true>},                              \
-     (int)((NW) * hj::Pf3Layout<float, LX, RY, RZ>::PER_WARP * sizeof(float)), {nullptr, nullptr}, 0, 0}
+     (int)((NW) * hj::Pf3Layout<float, LX, RY, RZ>::PER_WARP * sizeof(float)), {nullptr, nullptr}, 0, 0, 1}

@@ -463,6 +463,7 @@ struct Tile3Info {
     PpcKernel ppc[2];  // TMA-pipelined variant (binary32; null otherwise): one warp per CTA, dynamic smem ppc_smem
     int ppc_smem;
     int ppc_cps;       // its resident CTAs per SM unless the caller sets ctas_per_sm (0: as many as fit)
+    int ppc_ns;        // its subdomains along x per CTA (one warp each)
 };
 const Tile3Info *tiles3d_f64(int *n);
 const Tile3Info *tiles3d_f32(int *n);
