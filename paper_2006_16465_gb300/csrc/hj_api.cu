@@ -680,6 +680,7 @@ struct RunOut {
 struct ThirdBuffer {
     void **slot;
     size_t bytes;
+    int esz;       // element size
     void *alias;   // in-place runs: every iterate buffer is this array
 };
 
@@ -750,7 +751,7 @@ int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, 
             }
         }
         b2 = *third.slot;
-        CKR(cudaMemcpyAsync(b2, b0, third.bytes, cudaMemcpyDeviceToDevice, s));   // same ghost ring
+        CKR(launch_copy_ring(h->d.dim, third.esz, b0, b2, nullptr, base.ld, base.ps, h->d.nx, h->d.ny, h->d.nz, s));
     }
     Plan pl;
     CKS(make_plan(h, ki, pi, fam, classic, sig, true, base, b0, b1, b2, &pl));
@@ -912,10 +913,10 @@ int residual_of(hj_handle *h, const void *f, const void *u, bool transpose, doub
     const RedArgs red = red_args(h, RED_STORE, 0.0, 0);
     if (h->d.dim == 3)
         CKR(launch_residual3d(h->d.dtype == HJ_F64, f, u, h->d.ld, a.ps, h->d.nx, h->d.ny, h->d.nz, a.cW, a.cE,
-                              a.cS, a.cN, a.cB, a.cT, a.dconst, 1, red, s));
+                              a.cS, a.cN, a.cB, a.cT, a.dconst, ff ? 1 : 0, red, s));
     else
         CKR(launch_residual_ex(h->d.dim, h->d.dtype == HJ_F64, f, u, h->d.sigma, h->d.ld, h->d.ld, h->d.nx,
-                               h->d.ny, a.cW, a.cE, a.cS, a.cN, a.dconst, 1, nullptr, red, s, h->d.coef,
+                               h->d.ny, a.cW, a.cE, a.cS, a.cN, a.dconst, ff ? 1 : 0, nullptr, red, s, h->d.coef,
                                (long long)h->rows * h->d.ld));
     CKR(cudaMemcpyAsync(h->h_rstore, h->rstore, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
     CKR(cudaEventRecord(h->ev, s));
@@ -923,6 +924,19 @@ int residual_of(hj_handle *h, const void *f, const void *u, bool transpose, doub
     if (rr) *rr = h->h_rstore[0];
     if (ff) *ff = h->h_rstore[1];
     return HJ_OK;
+}
+
+// The second iterate buffer's ghost ring, and an iterate that ended in another
+// buffer back into the caller's array (padding columns stay the caller's).
+// Whole-array copies took 80 us (8192 x 8192 binary32) to 160 us (512^3) each.
+cudaError_t copy_ring(const hj_handle *h, const void *u, void *dst, cudaStream_t s) {
+    return launch_copy_ring(h->d.dim, (int)h->esz, u, dst, nullptr, h->d.ld, (long long)(h->d.ny + 2) * h->d.ld, h->d.nx,
+                            h->d.ny, h->d.nz, s);
+}
+cudaError_t copy_back(const hj_handle *h, void *u, const void *src, cudaStream_t s) {
+    const size_t pitch = (size_t)h->d.ld * h->esz;
+    return cudaMemcpy2DAsync(u, pitch, src, pitch, (size_t)(h->d.nx + 2) * h->esz, h->grid_bytes / pitch,
+                             cudaMemcpyDeviceToDevice, s);
 }
 
 // Plain (binary64 or binary32) solve of A u = f, u in/out (device).
@@ -934,7 +948,7 @@ int solve_plain(hj_handle *h, const void *f, void *u, bool transpose, cudaStream
     base.f = f;
     base.dinv = h->dinv_outer;
     const bool inplace = h->p.in_place != 0;
-    if (!inplace) CKR(cudaMemcpyAsync(h->ubuf, u, h->grid_bytes, cudaMemcpyDeviceToDevice, s));
+    if (!inplace) CKR(copy_ring(h, u, h->ubuf, s));
     // in place, even the first cycle's staged data may mix u_0 and u_1: take
     // ||r_0|| exactly for the final status
     double r0_exact = -1.0;
@@ -947,9 +961,9 @@ int solve_plain(hj_handle *h, const void *f, void *u, bool transpose, cudaStream
     long long hl = 0;
     int persist = 0;
     CKS(iterate(h, ki, classic ? nullptr : h->p_outer, h->fam_outer, classic, sig, base, u, inplace ? u : h->ubuf,
-                ThirdBuffer{&h->ubuf2, h->grid_bytes, inplace ? u : nullptr}, h->p.tol, h->p.max_cycles,
+                ThirdBuffer{&h->ubuf2, h->grid_bytes, (int)h->esz, inplace ? u : nullptr}, h->p.tol, h->p.max_cycles,
                 h->p.fixed_cycles, s, &ro, st ? st->history : nullptr, st ? st->history_cap : 0, &hl, &persist));
-    if (ro.buf != u) CKR(cudaMemcpyAsync(u, ro.buf, h->grid_bytes, cudaMemcpyDeviceToDevice, s));
+    if (ro.buf != u) CKR(copy_back(h, u, ro.buf, s));
     double res0 = -1.0, resc = -1.0;
     if (h->p.fixed_cycles <= 0) {
         res0 = inplace ? r0_exact : sqrt(std::max(ro.res2_0, 0.0));
@@ -990,7 +1004,7 @@ int solve_ir(hj_handle *h, const double *f, double *u, bool transpose, cudaStrea
     const CycArgs geo = base_args(h, transpose);
     const bool bf16 = h->fam_inner == FAM_BF16;
     const size_t dsz = bf16 ? 2 : 4;
-    CKR(cudaMemcpyAsync(h->ubuf, u, h->grid_bytes, cudaMemcpyDeviceToDevice, s));
+    CKR(copy_ring(h, u, h->ubuf, s));
     // outer residual of u_0 -> r32
     {
         const RedArgs red = red_args(h, RED_STORE, 0.0, 0);
@@ -1019,7 +1033,7 @@ int solve_ir(hj_handle *h, const double *f, double *u, bool transpose, cudaStrea
         RunOut ro;
         const bool inplace = h->p.in_place != 0;
         CKS(iterate(h, h->k_inner, h->p_inner, h->fam_inner, false, sig, base, h->dA, inplace ? h->dA : h->dB,
-                    ThirdBuffer{&h->dC, (size_t)h->rows * h->ld_in * dsz, inplace ? h->dA : nullptr},
+                    ThirdBuffer{&h->dC, (size_t)h->rows * h->ld_in * dsz, (int)dsz, inplace ? h->dA : nullptr},
                     h->p.inner_tol, h->p.inner_max_cycles, 0, s, &ro, nullptr, 0, nullptr, &persist));
         inner_total += ro.c;
         inner_launched += ro.launched;
@@ -1034,7 +1048,7 @@ int solve_ir(hj_handle *h, const double *f, double *u, bool transpose, cudaStrea
         rn = sqrt(h->h_rstore[0]);
         std::swap(cur, other);
     }
-    if (cur != u) CKR(cudaMemcpyAsync(u, cur, h->grid_bytes, cudaMemcpyDeviceToDevice, s));
+    if (cur != u) CKR(copy_back(h, u, cur, s));
     CKR(cudaStreamSynchronize(s));
     if (st) {
         st->cycles = inner_total;

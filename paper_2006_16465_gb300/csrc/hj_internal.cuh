@@ -503,6 +503,9 @@ cudaError_t launch_update_residual_ex(int dim, const double *f, const double *ui
                                       RedArgs red, cudaStream_t s);
 cudaError_t launch_grad_sigma_ex(int dim, int user_f64, const void *lam, const void *u, double *dsig, long long ld,
                                  int nx, int ny, int accumulate, cudaStream_t s);
+// the ghost ring (3D: shell) of src into d1 and, where not null, d2
+cudaError_t launch_copy_ring(int dim, int esz, const void *src, void *d1, void *d2, long long ld, long long ps, int nx,
+                             int ny, int nz, cudaStream_t s);
 int aux_max_blocks(int dim, int nx, int ny);
 int aux_sm_count();
 
