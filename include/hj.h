@@ -201,8 +201,10 @@ typedef struct {
                              i.e. the correction has reached the fixed point its
                              storage precision allows; 0 = off                 */
     int ctas_per_sm;      /* TMA-pipelined kernel: resident CTAs per SM (0 = as
-                             many as fit).  Fewer CTAs keep fewer copies in
-                             flight, which HBM can serve at a higher rate     */
+                             many as fit; fewer where binary32 grids larger
+                             than L2 are bound by HBM).  Fewer CTAs keep fewer
+                             copies in flight, which HBM can serve at a
+                             higher rate                                      */
     int overlap_x;        /* overlapping subdomains (Sections 3.4 and 4.3):
                              points shared by neighbouring subdomains along x
                              (0 <= overlap_x < tile_x).  Starts advance by
@@ -258,7 +260,7 @@ typedef struct {
     int tile_threads;         /* threads per subdomain actually used             */
     int persistent;           /* 1 if the persistent path ran                    */
     int pipeline_stages;      /* copy stages of the pipelined kernel if it runs, else 0 */
-    int ctas_per_sm;          /* its CTAs-per-SM cap (0 = as many as fit)         */
+    int ctas_per_sm;          /* its CTAs-per-SM cap (0 = the default)         */
     int overlap_x, overlap_y; /* overlapping points used (Sections 3.4, 4.3)      */
     int tile_z;               /* 3D: subdomain depth used (1 otherwise)           */
     /* hj_solve_batched / hj_solve_adjoint_batched: */

@@ -465,6 +465,22 @@ bool deferred_run(const hj_handle *h, const TileKernelInfo *ki, const PpcKernelI
 }
 
 
+// Resident CTAs per SM of the 2D pipelined kernel where the caller leaves the
+// choice.  HBM serves the box copies at its full rate up to about 93 KB of them
+// in flight per SM and more slowly beyond (8192 x 8192 binary32, us a cycle, at
+// full residency and at the cap: 32 x 32, 12 -> 10 CTAs: k = 1 136.6 -> 121.6,
+// k = 4 137.6 -> 122.5; 32 x 16, 22 -> 19: 132.5 -> 121, 128.7 -> 121; 64 x 32,
+// 6 -> 5: 131.8 -> 119.4, 130.3 -> 121.6).  Grids that L2 holds (3000 x 2000: no
+// difference at k = 1, 15.1 against 17.2 at k = 4) and cycles bound by their
+// sweeps (k = 5: 138 against 123, k = 6: 126 against 132, k = 16: 224 against
+// 255) want every warp that fits.
+int default_residency(const hj_handle *h, const PpcKernelInfo *pi, int fam, bool sig) {
+    if (fam != FAM_F32 || sig || pi->stages != 1 || h->p.k > 5) return 1 << 20;
+    if (3 * (long long)h->rows * h->d.ld * 4 <= (long long)h->l2_bytes) return 1 << 20;
+    const int flight = 4 * (pi->bwu * (pi->ty + 2) + pi->bwf * pi->ty);   // one CTA's copies, bytes
+    return std::max(1, 95 * 1024 / flight);
+}
+
 // b2: third iterate buffer (same ghost ring as b0), required when the
 // pipelined kernel runs with the fused residual.
 int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int fam, bool classic, bool sig,
@@ -620,6 +636,7 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
     CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, pi->threads, smem));
     if (occ < 1) return seterr(HJ_ERR_UNSUPPORTED, "pipelined kernel does not fit on an SM");
     if (h->p.ctas_per_sm > 0) occ = std::min(occ, h->p.ctas_per_sm);
+    else occ = std::min(occ, default_residency(h, pi, fam, sig));
     const int tiles_x = (nx + pi->tx - 1) / pi->tx;
     const int ntiles = tiles_x * ((ny + pi->ty - 1) / pi->ty);
     const int ssz = fam == FAM_F64 ? 8 : fam == FAM_BF16 ? 2 : 4;
@@ -1423,6 +1440,7 @@ int hj_create(hj_handle **out, const hj_desc *desc, const hj_params *params) {
     } while (0)
     if (cudaGetDevice(&h->dev) != cudaSuccess) HJ_FAIL(HJ_ERR_CUDA, "no CUDA device");
     cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->dev);
+    cudaDeviceGetAttribute(&h->l2_bytes, cudaDevAttrL2CacheSize, h->dev);
 
     h->ld_in = ((long long)d.nx + 2 + 31) / 32 * 32;
     // 1D with fewer subdomains than SMs: a cycle is the latency of one

@@ -312,12 +312,12 @@ int tune_launch(const hj_desc &d, hj_params *p) {
         }
         for (int c = occ; c >= std::max(1, occ / 2); --c) {
             double us = INFINITY;
-            if (!measure_launch(sc, prec, e.tx, e.ty, e.threads, e.stages, c == occ ? 0 : c, p->k, &us)) continue;
+            if (!measure_launch(sc, prec, e.tx, e.ty, e.threads, e.stages, c, p->k, &us)) continue;
             if (us < best) {
                 best = us;
                 bth = e.threads;
                 bst = e.stages;
-                bcps = c == occ ? 0 : c;
+                bcps = c;
             }
         }
     }

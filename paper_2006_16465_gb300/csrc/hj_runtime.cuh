@@ -74,7 +74,7 @@ struct MgLevel {
 struct hj_handle {
     hj_desc d;
     hj_params p;
-    int dev = 0, nsm = 0;
+    int dev = 0, nsm = 0, l2_bytes = 0;
     int rows = 0;
     size_t esz = 0, grid_elems = 0, grid_bytes = 0;
     int fam_outer = hj::FAM_F64, fam_inner = hj::FAM_F32;
