@@ -12,9 +12,10 @@
 //     up to four rows, the subdomain plus halo in two shared-memory
 //     containers, k damped Jacobi subiterations u' = u + omega (jac - u)
 //     with the halo frozen;
-//   * mg_restrict_kernel: the fine residual f - A u at the nine fine points
-//     around each coarse point, full-weighted into the coarse right-hand side
-//     (fused, no residual array), and the coarse correction set to zero;
+//   * mg_restrict_kernel (binary32), mg_restrict_tile_kernel (binary64): the fine
+//     residual f - A u at the nine fine points around each coarse point,
+//     full-weighted into the coarse right-hand side (fused, no residual array),
+//     and the coarse correction set to zero;
 //   * mg_prolong_kernel: u + bilinear interpolation of the coarse correction,
 //     one thread per coarse cell writing the 2 x 2 fine points inside it.
 // The graph also holds the residual norm of the level-0 iterate and its copy
@@ -46,7 +47,7 @@ struct MgXferArgs {
 
 // What a smoothing launch stages besides its level's iterate and RHS:
 //   MG_PLAIN:    u and f of the level;
-//   MG_RESTRICT: the level's first smoothing after the restriction: the RHS is
+//   MG_RESTRICT: (binary32) the level's first smoothing after the restriction: the RHS is
 //                the full-weighted fine residual (x: the finer level), formed
 //                here and also stored as the level's f, and the iterate (the
 //                coarse correction) starts at zero;
@@ -72,57 +73,59 @@ __device__ __forceinline__ T ld_g(const T *p) {
     return __ldg(p);
 }
 
-// f - A u at fine index q, in the oracle's order (binary64) or fused (binary32)
-template <typename T, bool EXACT>
-__device__ __forceinline__ T mg_resid(const MgXferArgs &x, const T *u, const T *f, long long q) {
-    if constexpr (EXACT) {
-        double au = __dmul_rn(x.d, u[q]);
-        au = __dadd_rn(au, __dmul_rn(x.cW, u[q - 1]));
-        au = __dadd_rn(au, __dmul_rn(x.cE, u[q + 1]));
-        au = __dadd_rn(au, __dmul_rn(x.cS, u[q - x.ld]));
-        au = __dadd_rn(au, __dmul_rn(x.cN, u[q + x.ld]));
-        return __dsub_rn(f[q], au);
-    } else {
-        T r = fmaf(-(T)x.d, u[q], f[q]);
-        r = fmaf(-(T)x.cW, u[q - 1], r);
-        r = fmaf(-(T)x.cE, u[q + 1], r);
-        r = fmaf(-(T)x.cS, u[q - x.ld], r);
-        r = fmaf(-(T)x.cN, u[q + x.ld], r);
-        return r;
-    }
+// whether two values differ in any bit
+__device__ __forceinline__ bool bits_differ(double x, double y) {
+    return __double_as_longlong(x) != __double_as_longlong(y);
+}
+__device__ __forceinline__ bool bits_differ(float x, float y) { return __float_as_uint(x) != __float_as_uint(y); }
+
+// x * 2^-n (n = 1, 2, ..), correctly rounded, by an integer subtraction in the
+// exponent field where x and the result are normal, else by the multiplication.
+template <int N>
+__device__ __forceinline__ double scale_down(double x) {
+    const int hi = __double2hiint(x);
+    const unsigned e = (unsigned)hi & 0x7ff00000u;
+    if (e - ((unsigned)(N + 1) << 20) < (0x7fe00000u - ((unsigned)N << 20)))
+        return __hiloint2double(hi - (N << 20), __double2loint(x));
+    return __dmul_rn(x, 1.0 / (1 << N));
 }
 
-// The full-weighted fine residual at coarse point (I, J): the restriction.
-template <typename T, bool EXACT>
-__device__ __forceinline__ T restrict_at(const MgXferArgs &x, int I, int J) {
-    const T *u = (const T *)x.u, *f = (const T *)x.f;
+// x * c, correctly rounded, on the integer pipes where they cover it (mul_const)
+__device__ __forceinline__ double mul_rn(double x, const MulConst &m, double c) {
+    unsigned bad = 0;
+    double r = mul_const(x, m, bad);
+    if (bad > m.span) r = __dmul_rn(x, c);
+    return r;
+}
+
+// Binary32: f - A u at fine index q as a fused chain
+__device__ __forceinline__ float mg_resid(const MgXferArgs &x, const float *u, const float *f, long long q) {
+    float r = fmaf(-(float)x.d, u[q], f[q]);
+    r = fmaf(-(float)x.cW, u[q - 1], r);
+    r = fmaf(-(float)x.cE, u[q + 1], r);
+    r = fmaf(-(float)x.cS, u[q - x.ld], r);
+    r = fmaf(-(float)x.cN, u[q + x.ld], r);
+    return r;
+}
+
+// Binary32: the full-weighted fine residual at coarse point (I, J), the restriction
+// (binary64: mg_restrict_tile_kernel).
+__device__ __forceinline__ float restrict_at(const MgXferArgs &x, int I, int J) {
+    const float *u = (const float *)x.u, *f = (const float *)x.f;
     const long long q = 2LL * J * x.ld + 2LL * I, ld = x.ld;
-    const T r00 = mg_resid<T, EXACT>(x, u, f, q);
-    if constexpr (EXACT) {
-        double s1 = __dadd_rn(mg_resid<T, EXACT>(x, u, f, q - 1), mg_resid<T, EXACT>(x, u, f, q + 1));
-        s1 = __dadd_rn(s1, mg_resid<T, EXACT>(x, u, f, q - ld));
-        s1 = __dadd_rn(s1, mg_resid<T, EXACT>(x, u, f, q + ld));
-        double s2 = __dadd_rn(mg_resid<T, EXACT>(x, u, f, q - ld - 1), mg_resid<T, EXACT>(x, u, f, q - ld + 1));
-        s2 = __dadd_rn(s2, mg_resid<T, EXACT>(x, u, f, q + ld - 1));
-        s2 = __dadd_rn(s2, mg_resid<T, EXACT>(x, u, f, q + ld + 1));
-        double t = __dmul_rn(4.0, r00);
-        t = __dadd_rn(t, __dmul_rn(2.0, s1));
-        t = __dadd_rn(t, s2);
-        return __dmul_rn(t, 0.0625);
-    } else {
-        const T s1 = (mg_resid<T, EXACT>(x, u, f, q - 1) + mg_resid<T, EXACT>(x, u, f, q + 1)) +
-                     (mg_resid<T, EXACT>(x, u, f, q - ld) + mg_resid<T, EXACT>(x, u, f, q + ld));
-        const T s2 = (mg_resid<T, EXACT>(x, u, f, q - ld - 1) + mg_resid<T, EXACT>(x, u, f, q - ld + 1)) +
-                     (mg_resid<T, EXACT>(x, u, f, q + ld - 1) + mg_resid<T, EXACT>(x, u, f, q + ld + 1));
-        return (4.0f * r00 + 2.0f * s1 + s2) * 0.0625f;
-    }
+    const float r00 = mg_resid(x, u, f, q);
+    const float s1 = (mg_resid(x, u, f, q - 1) + mg_resid(x, u, f, q + 1)) +
+                     (mg_resid(x, u, f, q - ld) + mg_resid(x, u, f, q + ld));
+    const float s2 = (mg_resid(x, u, f, q - ld - 1) + mg_resid(x, u, f, q - ld + 1)) +
+                     (mg_resid(x, u, f, q + ld - 1) + mg_resid(x, u, f, q + ld + 1));
+    return (4.0f * r00 + 2.0f * s1 + s2) * 0.0625f;
 }
 
 // Bilinear interpolation of the coarse correction: a fine point between four
 // coarse points (both indices odd), between two (one odd), or on one.
 template <typename T, bool EXACT>
 __device__ __forceinline__ T avg2(T x, T y) {
-    if constexpr (EXACT) return __dmul_rn(__dadd_rn(x, y), 0.5);
+    if constexpr (EXACT) return scale_down<1>(__dadd_rn(x, y));
     else return (x + y) * (T)0.5;
 }
 
@@ -132,7 +135,7 @@ __device__ __forceinline__ T avg4(T e00, T e10, T e01, T e11) {
         double t = __dadd_rn(e00, e10);
         t = __dadd_rn(t, e01);
         t = __dadd_rn(t, e11);
-        return __dmul_rn(t, 0.25);
+        return scale_down<2>(t);
     } else {
         return ((e00 + e10) + (e01 + e11)) * (T)0.25;
     }
@@ -154,6 +157,13 @@ __device__ __forceinline__ T prolong_at(const MgXferArgs &x, int i, int j) {
     if (j & 1) {
         const T *r1 = r0 + ldc;
         const T e00 = r0[cl], e10 = r0[cr], e01 = r1[cl], e11 = r1[cr];
+        if constexpr (EXACT) {
+            // both parities from one chain of sums (avg2 is its first, avg4 all three)
+            const double t1 = __dadd_rn(e00, odd_i ? e10 : e01);
+            const double t3 = __dadd_rn(__dadd_rn(t1, e01), e11);
+            const double v2 = scale_down<1>(t1), v4 = scale_down<2>(t3);
+            return odd_i ? v4 : v2;
+        }
         const T vo = avg4<T, EXACT>(e00, e10, e01, e11), ve = avg2<T, EXACT>(e00, e01);
         return odd_i ? vo : ve;
     }
@@ -195,12 +205,22 @@ __global__ void __launch_bounds__(1024 / RPT, (RPT == 1 && STAGE == MG_PLAIN) ? 
         const int j = j0 + ty + m * BY;
         in[m] = i <= nx && j <= ny;
         v0[m] = ld_u(j, i);
-        hw[m] = tx == 0 ? ld_u(j, i - 1) : (T)0;
-        he[m] = tx == TX - 1 ? ld_u(j, i + 1) : (T)0;
+        if constexpr (EXACT && stage == MG_PROLONG) {
+            // one call for both edge columns: here each is binary64 work for the whole warp
+            hw[m] = he[m] = (T)0;
+            if (tx == 0 || tx == TX - 1) {
+                const T h = ld_u(j, tx == 0 ? i - 1 : i + 1);
+                if (tx == 0) hw[m] = h;
+                if (tx == TX - 1) he[m] = TX == 1 ? ld_u(j, i + 1) : h;
+            }
+        } else {
+            hw[m] = tx == 0 ? ld_u(j, i - 1) : (T)0;
+            he[m] = tx == TX - 1 ? ld_u(j, i + 1) : (T)0;
+        }
         T fv = (T)0;
         if (in[m]) {
-            if (stage == MG_RESTRICT) {
-                fv = restrict_at<T, EXACT>(a.x, i, j);
+            if constexpr (stage == MG_RESTRICT) {
+                fv = restrict_at(a.x, i, j);
                 ((T *)a.x.fc)[(long long)j * ld + i] = fv;
             } else {
                 fv = ld_g((const T *)a.f + (long long)j * ld + i);
@@ -218,10 +238,19 @@ __global__ void __launch_bounds__(1024 / RPT, (RPT == 1 && STAGE == MG_PLAIN) ? 
     // 1e-8: 5.94 -> 5.30 ms).  Otherwise they hold the values.
     bool share = false;
     if constexpr (EXACT) share = same_bits(a.cW, a.cE) && same_bits(a.cS, a.cN) && same_bits(a.cW, a.cS);
+    // The three products by constants of a shared update (c u, (f - sum)/d and the
+    // damping) run on the integer pipes; a thread that meets a value they do not
+    // cover repeats its points on the FP64 pipe (mul_const: 9 become 6 there).
     auto run = [&](auto share_tag) {
         constexpr bool SH = decltype(share_tag)::value;
+        MulConst mc, mi, mo;
+        if constexpr (SH) {
+            mc = make_mul_const(a.cW);
+            mi = make_mul_const(a.invd);
+            mo = make_mul_const(a.omega);
+        }
         auto term = [&](T v) -> T {
-            if constexpr (SH) return (T)__dmul_rn(a.cW, v);
+            if constexpr (SH) return (T)mul_rn(v, mc, a.cW);
             else return v;
         };
 #pragma unroll
@@ -236,43 +265,84 @@ __global__ void __launch_bounds__(1024 / RPT, (RPT == 1 && STAGE == MG_PLAIN) ? 
         if (ty == 0) { const T w = term(hs); buf0[tx + 1] = w; buf1[tx + 1] = w; }
         if (ty == BY - 1) { const T w = term(hn); buf0[(TY + 1) * lw + tx + 1] = w; buf1[(TY + 1) * lw + tx + 1] = w; }
         __syncthreads();
+        // one point from its neighbours' terms; INT: collects in bad what it cannot do
+        auto update = [&](int m, const T *src, auto int_tag, T &prod, unsigned &bad) -> T {
+            constexpr bool INT = decltype(int_tag)::value;
+            const int me = (ty + m * BY + 1) * lw + tx + 1;
+            const T old = v0[m];
+            const T W = src[me - 1], E = src[me + 1], Sv = src[me - lw], Nv = src[me + lw];
+            T nv;
+            if constexpr (EXACT) {
+                double acc;
+                if constexpr (SH) {
+                    acc = __dadd_rn(W, E);
+                    acc = __dadd_rn(acc, Sv);
+                    acc = __dadd_rn(acc, Nv);
+                } else {
+                    acc = __dmul_rn(a.cW, W);
+                    acc = __dadd_rn(acc, __dmul_rn(a.cE, E));
+                    acc = __dadd_rn(acc, __dmul_rn(a.cS, Sv));
+                    acc = __dadd_rn(acc, __dmul_rn(a.cN, Nv));
+                }
+                const double t = __dsub_rn(g[m], acc);
+                if constexpr (INT) {
+                    unsigned b0 = 0, b1 = 0, b2 = 0;
+                    const double jac = mul_const(t, mi, b0);
+                    nv = __dadd_rn(old, mul_const(__dsub_rn(jac, old), mo, b1));
+                    prod = mul_const(nv, mc, b2);
+                    bad |= (unsigned)(b0 > mi.span) | (unsigned)(b1 > mo.span) | (unsigned)(b2 > mc.span);
+                } else {
+                    const double jac = __dmul_rn(t, a.invd);
+                    nv = __dadd_rn(old, __dmul_rn(a.omega, __dsub_rn(jac, old)));
+                    prod = SH ? __dmul_rn(a.cW, nv) : nv;
+                }
+            } else {
+                T t = g[m];
+                t = fmaf(a.fN, Nv, t);
+                t = fmaf(a.fS, Sv, t);
+                t = fmaf(a.fE, E, t);
+                t = fmaf(a.fW, W, t);
+                nv = fmaf(a.fomega, t - old, old);
+                prod = nv;
+            }
+            return nv;
+        };
+        // Long runs (the coarsest level's) end at their fixed point: once a
+        // subiteration leaves every value as it was, bit for bit, so do all that
+        // follow.  A level of one point is there after two of its 256 (79 us of a
+        // V-cycle in binary64).
+        const bool watch = a.k >= 16;
         for (int s = 0; s < a.k; ++s) {
             const T *src = (s & 1) ? buf1 : buf0;
             T *dst = (s & 1) ? buf0 : buf1;
             const bool more = s + 1 < a.k;   // the last subiteration's values go to global memory from registers
+            T nv[RPT], prod[RPT];
+            unsigned bad = 0;
+#pragma unroll
+            for (int m = 0; m < RPT; ++m) {
+                unsigned b = 0;
+                nv[m] = update(m, src, std::integral_constant<bool, SH>(), prod[m], b);
+                if (in[m]) bad |= b;
+            }
+            if constexpr (SH) {
+                if (bad) {
+#pragma unroll
+                    for (int m = 0; m < RPT; ++m)
+                        nv[m] = update(m, src, std::integral_constant<bool, false>(), prod[m], bad);
+                }
+            }
+            bool changed = false;
 #pragma unroll
             for (int m = 0; m < RPT; ++m) {
                 if (!in[m]) continue;
-                const int me = (ty + m * BY + 1) * lw + tx + 1;
-                const T old = v0[m];
-                const T W = src[me - 1], E = src[me + 1], Sv = src[me - lw], Nv = src[me + lw];
-                T nv;
-                if constexpr (EXACT) {
-                    double acc;
-                    if constexpr (SH) {
-                        acc = __dadd_rn(W, E);
-                        acc = __dadd_rn(acc, Sv);
-                        acc = __dadd_rn(acc, Nv);
-                    } else {
-                        acc = __dmul_rn(a.cW, W);
-                        acc = __dadd_rn(acc, __dmul_rn(a.cE, E));
-                        acc = __dadd_rn(acc, __dmul_rn(a.cS, Sv));
-                        acc = __dadd_rn(acc, __dmul_rn(a.cN, Nv));
-                    }
-                    const double jac = __dmul_rn(__dsub_rn(g[m], acc), a.invd);
-                    nv = __dadd_rn(old, __dmul_rn(a.omega, __dsub_rn(jac, old)));
-                } else {
-                    T t = g[m];
-                    t = fmaf(a.fN, Nv, t);
-                    t = fmaf(a.fS, Sv, t);
-                    t = fmaf(a.fE, E, t);
-                    t = fmaf(a.fW, W, t);
-                    nv = fmaf(a.fomega, t - old, old);
-                }
-                v0[m] = nv;
-                if (more) dst[me] = term(nv);
+                changed = changed || bits_differ(nv[m], v0[m]);
+                v0[m] = nv[m];
+                if (more) dst[(ty + m * BY + 1) * lw + tx + 1] = prod[m];
             }
-            if (more) __syncthreads();
+            if (more) {
+                if (!watch) __syncthreads();
+                else if (!__syncthreads_or(changed)) break;
+            }
         }
     };
     if constexpr (EXACT) {
@@ -288,13 +358,73 @@ __global__ void __launch_bounds__(1024 / RPT, (RPT == 1 && STAGE == MG_PLAIN) ? 
     }
 }
 
-template <typename T, bool EXACT>
 __global__ void __launch_bounds__(256) mg_restrict_kernel(const MgXferArgs x) {
     const int I = 1 + blockIdx.x * 32 + threadIdx.x, J = 1 + blockIdx.y * 8 + threadIdx.y;
     if (I > x.ncx || J > x.ncy) return;
     const long long qc = (long long)J * x.ldc + I;
-    ((T *)x.fc)[qc] = restrict_at<T, EXACT>(x, I, J);
-    ((T *)x.ec)[qc] = (T)0;
+    ((float *)x.fc)[qc] = restrict_at(x, I, J);
+    ((float *)x.ec)[qc] = 0.f;
+}
+
+// Binary64 restriction of a block of 32 x 8 coarse points: the 65 x 17 fine
+// residuals around them are formed once each in shared memory and weighted from
+// there.  A thread per coarse point (the binary32 kernel above) forms nine residuals of ten operations per coarse
+// point; each fine one is needed 2.25 times on average, so on the FP64 pipe, which
+// bounds both, 104 operations a coarse point become some 50 (30 with the products
+// by constants, shared between neighbours where the coefficients are equal, on
+// the integer pipes).  Sums in restrict_at's order; 4 r + 2 s + t with exact
+// powers of two is 2 (2 r + s) + t, two fused operations with the same roundings.
+// 4095 x 4095 fine points: 330 us, and a coarse level's launch 5 to 10 us, where
+// forming nine residuals a point inside the next smoothing made that 13 us.
+__global__ void __launch_bounds__(256) mg_restrict_tile_kernel(const MgXferArgs x) {
+    constexpr int BW = 32, BH = 8, RW = 2 * BW + 1, RH = 2 * BH + 1, UW = RW + 2, UH = RH + 2;
+    __shared__ double U[UH][UW], P[UH][UW];   // u and c u on the residuals' points and one around
+    __shared__ double R[RH][RW + 1];
+    const double *u = (const double *)x.u, *f = (const double *)x.f;
+    const int I0 = 1 + blockIdx.x * BW, J0 = 1 + blockIdx.y * BH;
+    const int fx = 2 * I0 - 2, fy = 2 * J0 - 2;   // fine point of U[0][0]
+    const int tid = threadIdx.x + 32 * threadIdx.y;
+    const bool iso = same_bits(x.cW, x.cE) && same_bits(x.cS, x.cN) && same_bits(x.cW, x.cS);
+    const MulConst mc = make_mul_const(x.cW), md = make_mul_const(x.d);
+    for (int t = tid; t < UW * UH; t += 256) {
+        const int c = t % UW, r = t / UW;
+        double v = 0.0;
+        if (fx + c <= x.nx + 1 && fy + r <= x.ny + 1) v = u[(long long)(fy + r) * x.ld + fx + c];
+        U[r][c] = v;
+        if (iso) P[r][c] = mul_rn(v, mc, x.cW);
+    }
+    __syncthreads();
+    for (int t = tid; t < RW * RH; t += 256) {
+        const int c = t % RW, r = t / RW, gx = fx + 1 + c, gy = fy + 1 + r;
+        if (gx > x.nx || gy > x.ny) continue;   // (no coarse point here has such a neighbour)
+        double au = mul_rn(U[r + 1][c + 1], md, x.d);
+        if (iso) {
+            au = __dadd_rn(au, P[r + 1][c]);
+            au = __dadd_rn(au, P[r + 1][c + 2]);
+            au = __dadd_rn(au, P[r][c + 1]);
+            au = __dadd_rn(au, P[r + 2][c + 1]);
+        } else {
+            au = __dadd_rn(au, __dmul_rn(x.cW, U[r + 1][c]));
+            au = __dadd_rn(au, __dmul_rn(x.cE, U[r + 1][c + 2]));
+            au = __dadd_rn(au, __dmul_rn(x.cS, U[r][c + 1]));
+            au = __dadd_rn(au, __dmul_rn(x.cN, U[r + 2][c + 1]));
+        }
+        R[r][c] = __dsub_rn(f[(long long)gy * x.ld + gx], au);
+    }
+    __syncthreads();
+    const int I = I0 + (int)threadIdx.x, J = J0 + (int)threadIdx.y;
+    if (I > x.ncx || J > x.ncy) return;
+    const int c = 2 * threadIdx.x + 1, r = 2 * threadIdx.y + 1;   // R of fine point (2I, 2J)
+    double s1 = __dadd_rn(R[r][c - 1], R[r][c + 1]);
+    s1 = __dadd_rn(s1, R[r - 1][c]);
+    s1 = __dadd_rn(s1, R[r + 1][c]);
+    double s2 = __dadd_rn(R[r - 1][c - 1], R[r - 1][c + 1]);
+    s2 = __dadd_rn(s2, R[r + 1][c - 1]);
+    s2 = __dadd_rn(s2, R[r + 1][c + 1]);
+    const double t = __fma_rn(2.0, __fma_rn(2.0, R[r][c], s1), s2);
+    const long long qc = (long long)J * x.ldc + I;
+    ((double *)x.fc)[qc] = scale_down<4>(t);
+    ((double *)x.ec)[qc] = 0.0;
 }
 
 // One thread per coarse cell (a, b), a in [0, ncx], b in [0, ncy]: the fine
@@ -356,9 +486,12 @@ void launch_smooth(hj_handle *h, int l, int cur, int tx, int ty, int k, double o
         a.x = *x;
     }
     // rows per thread: 4 (or 2) when the subdomain height allows, 1 otherwise
-    const int rpt = (ty % 4 == 0 && ty >= 8) ? 4 : (ty % 2 == 0 && ty >= 4) ? 2 : 1;
-    const dim3 block(tx, ty / rpt), grid((L.nx + tx - 1) / tx, (L.ny + ty - 1) / ty);
     const bool f64 = h->fam_outer == FAM_F64;
+    int rpt = (ty % 4 == 0 && ty >= 8) ? 4 : (ty % 2 == 0 && ty >= 4) ? 2 : 1;
+    // binary64 is bound by the FP64 pipes, one per sub-partition: at least four
+    // warps a CTA before rows are added to a thread
+    while (f64 && rpt > 1 && tx * (ty / rpt) < 128) rpt /= 2;
+    const dim3 block(tx, ty / rpt), grid((L.nx + tx - 1) / tx, (L.ny + ty - 1) / ty);
     const int smem = 2 * (tx + 2) * (ty + 2) * (f64 ? 8 : 4);
 #define HJ_MG_SMOOTH(T, EX, ST)                                                            \
     do {                                                                                   \
@@ -368,11 +501,11 @@ void launch_smooth(hj_handle *h, int l, int cur, int tx, int ty, int k, double o
     } while (0)
 #define HJ_MG_SMOOTH_ST(T, EX)                                        \
     do {                                                              \
-        if (a.stage == MG_RESTRICT) HJ_MG_SMOOTH(T, EX, MG_RESTRICT); \
-        else if (a.stage == MG_PROLONG) HJ_MG_SMOOTH(T, EX, MG_PROLONG); \
+        if (a.stage == MG_PROLONG) HJ_MG_SMOOTH(T, EX, MG_PROLONG); \
         else HJ_MG_SMOOTH(T, EX, MG_PLAIN);                           \
     } while (0)
     if (f64) HJ_MG_SMOOTH_ST(double, true);
+    else if (a.stage == MG_RESTRICT) HJ_MG_SMOOTH(float, false, MG_RESTRICT);   // (binary32 only, record_level)
     else HJ_MG_SMOOTH_ST(float, false);
 #undef HJ_MG_SMOOTH_ST
 #undef HJ_MG_SMOOTH
@@ -397,8 +530,8 @@ constexpr long long kMgFuseMaxPoints = 512LL * 512;
 
 void launch_restrict(const hj_handle *h, const MgXferArgs &x, int ncx, int ncy, cudaStream_t s) {
     const dim3 g((ncx + 31) / 32, (ncy + 7) / 8), b(32, 8);
-    if (h->fam_outer == FAM_F64) mg_restrict_kernel<double, true><<<g, b, 0, s>>>(x);
-    else mg_restrict_kernel<float, false><<<g, b, 0, s>>>(x);
+    if (h->fam_outer == FAM_F64) mg_restrict_tile_kernel<<<g, b, 0, s>>>(x);
+    else mg_restrict_kernel<<<g, b, 0, s>>>(x);
 }
 
 // The V-cycle below level l, starting from buffer cur of level l; returns the
@@ -428,7 +561,10 @@ int record_level(hj_handle *h, int l, int cur, cudaStream_t s, const MgXferArgs 
             return cur;
         }
         if (l > 0) {
-            launch_smooth(h, l, cur, L.nx, L.ny, p.mg_coarse_k * p.mg_coarse_cycles, 1.0, s, MG_RESTRICT, rin);
+            const bool own = h->fam_outer == FAM_F64;   // its own restriction launch
+            if (own) launch_restrict(h, *rin, L.nx, L.ny, s);
+            launch_smooth(h, l, cur, L.nx, L.ny, p.mg_coarse_k * p.mg_coarse_cycles, 1.0, s, MG_RESTRICT,
+                          own ? nullptr : rin);
             return cur ^ 1;
         }
         for (int c = 0; c < p.mg_coarse_cycles; ++c) {
@@ -439,7 +575,9 @@ int record_level(hj_handle *h, int l, int cur, cudaStream_t s, const MgXferArgs 
     }
     const bool small = (long long)L.nx * L.ny <= kMgFuseMaxPoints;
     const MgXferArgs *pending = rin;
-    if (pending && (!small || p.mg_pre == 0)) {
+    // (binary64: forming nine residuals per point in the smoother's staging costs
+    // more FP64 time than the tiled restriction's launch: see mg_restrict_tile_kernel)
+    if (pending && (!small || p.mg_pre == 0 || h->fam_outer == FAM_F64)) {
         launch_restrict(h, *pending, L.nx, L.ny, s);
         pending = nullptr;
     }
