@@ -366,6 +366,69 @@ __global__ void __launch_bounds__(256) mg_restrict_kernel(const MgXferArgs x) {
     ((float *)x.ec)[qc] = 0.f;
 }
 
+// Binary32 smoothing of subdomains 32 columns wide and 4, 8, .. 32 high: a warp owns
+// four rows, a lane one column of them, in registers; W/E neighbours come by
+// shuffle and only the warps' edge rows pass through shared memory (as in
+// vc2d_rows_kernel; the sums are those of mg_smooth_kernel, bit for bit).  Bound by
+// HBM on the fine levels: 4095 x 4095, 32 x 8, k = 2
+// 57.8 -> 50.6 us.
+__global__ void __launch_bounds__(256) mg_smooth_rows_kernel(const MgSmoothArgs a) {
+    constexpr int R = 4;
+    constexpr unsigned ALL = 0xffffffffu;
+    __shared__ float edge[2][8][2][32];   // [parity][warp][first, last row][column]
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nx = a.nx, ny = a.ny;
+    const long long ld = a.ld;
+    const int i = 1 + blockIdx.x * 32 + lane, j0 = 1 + (blockIdx.y * nw + w) * R;
+    const float *__restrict__ u = (const float *)a.uin, *__restrict__ f = (const float *)a.f;
+    auto ld_u = [&](int jj, int ii) -> float {
+        return ii <= nx + 1 && jj <= ny + 1 ? __ldg(u + (long long)jj * ld + ii) : 0.f;
+    };
+    const bool edge_lane = lane == 0 || lane == 31;
+    float v[R], hx[R], g[R];
+    bool in[R];
+    float top = ld_u(j0 - 1, i), bot = ld_u(j0 + R, i);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int j = j0 + r;
+        in[r] = i <= nx && j <= ny;
+        v[r] = ld_u(j, i);
+        hx[r] = edge_lane ? ld_u(j, lane == 0 ? i - 1 : i + 1) : 0.f;
+        g[r] = in[r] ? __ldg(f + (long long)j * ld + i) : 0.f;
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) g[r] = g[r] * a.finvd;
+    for (int s = 0; s < a.k; ++s) {
+        float prev = top;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float cur = v[r];
+            float W = __shfl_up_sync(ALL, cur, 1), E = __shfl_down_sync(ALL, cur, 1);
+            if (lane == 0) W = hx[r];
+            if (lane == 31) E = hx[r];
+            float t = g[r];
+            t = fmaf(a.fN, r < R - 1 ? v[r < R - 1 ? r + 1 : 0] : bot, t);
+            t = fmaf(a.fS, prev, t);
+            t = fmaf(a.fE, E, t);
+            t = fmaf(a.fW, W, t);
+            v[r] = in[r] ? fmaf(a.fomega, t - cur, cur) : cur;
+            prev = cur;
+        }
+        if (nw > 1 && s + 1 < a.k) {
+            const int par = s & 1;
+            edge[par][w][0][lane] = v[0];
+            edge[par][w][1][lane] = v[R - 1];
+            __syncthreads();
+            if (w > 0) top = edge[par][w - 1][1][lane];
+            if (w < nw - 1) bot = edge[par][w + 1][0][lane];
+        }
+    }
+    float *__restrict__ uo = (float *)a.uout;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if (in[r]) uo[(long long)(j0 + r) * ld + i] = v[r];
+}
+
 // Binary64 restriction of a block of 32 x 8 coarse points: the 65 x 17 fine
 // residuals around them are formed once each in shared memory and weighted from
 // there.  A thread per coarse point (the binary32 kernel above) forms nine residuals of ten operations per coarse
@@ -374,8 +437,8 @@ __global__ void __launch_bounds__(256) mg_restrict_kernel(const MgXferArgs x) {
 // by constants, shared between neighbours where the coefficients are equal, on
 // the integer pipes).  Sums in restrict_at's order; 4 r + 2 s + t with exact
 // powers of two is 2 (2 r + s) + t, two fused operations with the same roundings.
-// 4095 x 4095 fine points: 330 us, and a coarse level's launch 5 to 10 us, where
-// forming nine residuals a point inside the next smoothing made that 13 us.
+// 4095 x 4095 fine points: 327 us; a coarse level's launch 4 to 7 us, where forming
+// nine residuals a point inside the next smoothing made that launch 13 us longer.
 __global__ void __launch_bounds__(256) mg_restrict_tile_kernel(const MgXferArgs x) {
     constexpr int BW = 32, BH = 8, RW = 2 * BW + 1, RH = 2 * BH + 1, UW = RW + 2, UH = RH + 2;
     __shared__ double U[UH][UW], P[UH][UW];   // u and c u on the residuals' points and one around
@@ -386,17 +449,34 @@ __global__ void __launch_bounds__(256) mg_restrict_tile_kernel(const MgXferArgs 
     const int tid = threadIdx.x + 32 * threadIdx.y;
     const bool iso = same_bits(x.cW, x.cE) && same_bits(x.cS, x.cN) && same_bits(x.cW, x.cS);
     const MulConst mc = make_mul_const(x.cW), md = make_mul_const(x.d);
-    for (int t = tid; t < UW * UH; t += 256) {
-        const int c = t % UW, r = t / UW;
-        double v = 0.0;
-        if (fx + c <= x.nx + 1 && fy + r <= x.ny + 1) v = u[(long long)(fy + r) * x.ld + fx + c];
-        U[r][c] = v;
-        if (iso) P[r][c] = mul_rn(v, mc, x.cW);
+    // every load first: one round of memory latency per CTA, which is most of what
+    // a coarse level's launch costs
+    constexpr int NU = (UW * UH + 255) / 256, NR = (RW * RH + 255) / 256;
+    double uv[NU], fv[NR];
+#pragma unroll
+    for (int k = 0; k < NU; ++k) {
+        const int t = tid + 256 * k, c = t % UW, r = t / UW;
+        uv[k] = 0.0;
+        if (t < UW * UH && fx + c <= x.nx + 1 && fy + r <= x.ny + 1) uv[k] = __ldg(u + (long long)(fy + r) * x.ld + fx + c);
+    }
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+        const int t = tid + 256 * k, gx = fx + 1 + t % RW, gy = fy + 1 + t / RW;
+        fv[k] = 0.0;
+        if (t < RW * RH && gx <= x.nx && gy <= x.ny) fv[k] = __ldg(f + (long long)gy * x.ld + gx);
+    }
+#pragma unroll
+    for (int k = 0; k < NU; ++k) {
+        const int t = tid + 256 * k, c = t % UW, r = t / UW;
+        if (t >= UW * UH) continue;
+        U[r][c] = uv[k];
+        if (iso) P[r][c] = mul_rn(uv[k], mc, x.cW);
     }
     __syncthreads();
-    for (int t = tid; t < RW * RH; t += 256) {
-        const int c = t % RW, r = t / RW, gx = fx + 1 + c, gy = fy + 1 + r;
-        if (gx > x.nx || gy > x.ny) continue;   // (no coarse point here has such a neighbour)
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+        const int t = tid + 256 * k, c = t % RW, r = t / RW;
+        if (t >= RW * RH || fx + 1 + c > x.nx || fy + 1 + r > x.ny) continue;   // (no coarse point here has such a neighbour)
         double au = mul_rn(U[r + 1][c + 1], md, x.d);
         if (iso) {
             au = __dadd_rn(au, P[r + 1][c]);
@@ -409,7 +489,7 @@ __global__ void __launch_bounds__(256) mg_restrict_tile_kernel(const MgXferArgs 
             au = __dadd_rn(au, __dmul_rn(x.cS, U[r][c + 1]));
             au = __dadd_rn(au, __dmul_rn(x.cN, U[r + 2][c + 1]));
         }
-        R[r][c] = __dsub_rn(f[(long long)gy * x.ld + gx], au);
+        R[r][c] = __dsub_rn(fv[k], au);
     }
     __syncthreads();
     const int I = I0 + (int)threadIdx.x, J = J0 + (int)threadIdx.y;
@@ -427,9 +507,12 @@ __global__ void __launch_bounds__(256) mg_restrict_tile_kernel(const MgXferArgs 
     ((double *)x.ec)[qc] = 0.0;
 }
 
-// One thread per coarse cell (a, b), a in [0, ncx], b in [0, ncy]: the fine
-// points (2a+1 | 2a+2, 2b+1 | 2b+2) inside it, each with the oracle's formula
-// for its parity; a warp writes coalesced pairs of every fine row.
+// One thread per coarse cell (ca, cb), ca in [0, ncx], cb in [0, ncy]: the fine
+// points (2ca | 2ca+1, 2cb | 2cb+1), each with the oracle's formula for its parity
+// (row and column 0 are ghosts and left alone).  The two points of a row are one
+// aligned vector, so a warp reads and writes whole lines of every fine row (as
+// the cell's inner points, 2ca+1 | 2ca+2, they were two strided halves: 4095 x
+// 4095 binary32 58.8 -> 25.3 us; binary64, bound by its sums, 100 -> 107).
 template <typename T, bool EXACT>
 __global__ void __launch_bounds__(256) mg_prolong_kernel(const MgXferArgs x) {
     const int ca = blockIdx.x * 32 + threadIdx.x, cb = blockIdx.y * 8 + threadIdx.y;
@@ -437,19 +520,23 @@ __global__ void __launch_bounds__(256) mg_prolong_kernel(const MgXferArgs x) {
     const T *e = (const T *)x.ec;
     const long long r0 = (long long)cb * x.ldc, r1 = r0 + x.ldc;
     const T e00 = e[r0 + ca], e10 = e[r0 + ca + 1], e01 = e[r1 + ca], e11 = e[r1 + ca + 1];
-    const int i1 = 2 * ca + 1, j1 = 2 * cb + 1;
-    const bool xe = ca < x.ncx, ye = cb < x.ncy;   // the even column / row exists
-    const T *ui = (const T *)x.u;
-    T *uo = (T *)x.uout;
-    auto put = [&](int ii, int jj, T v) {
-        const long long q = (long long)jj * x.ld + ii;
-        const T un = ui[q];
-        uo[q] = EXACT ? (T)__dadd_rn(un, v) : un + v;
+    struct alignas(2 * sizeof(T)) Pair {
+        T x, y;
     };
-    put(i1, j1, avg4<T, EXACT>(e00, e10, e01, e11));             // (odd, odd)
-    if (xe) put(i1 + 1, j1, avg2<T, EXACT>(e10, e11));          // (even, odd)
-    if (ye) put(i1, j1 + 1, avg2<T, EXACT>(e01, e11));          // (odd, even)
-    if (xe && ye) put(i1 + 1, j1 + 1, e11);                     // (even, even)
+    auto add = [](T u, T v) -> T { return EXACT ? (T)__dadd_rn(u, v) : u + v; };
+    auto put = [&](int jj, T ve, T vo) {   // corrections of the row's even and odd column
+        const long long q = (long long)jj * x.ld + 2 * ca;
+        const T *ui = (const T *)x.u + q;
+        T *uo = (T *)x.uout + q;
+        if (ca > 0) {
+            const Pair u = *(const Pair *)ui;
+            *(Pair *)uo = Pair{add(u.x, ve), add(u.y, vo)};
+        } else {
+            uo[1] = add(ui[1], vo);
+        }
+    };
+    if (cb > 0) put(2 * cb, e00, avg2<T, EXACT>(e00, e10));
+    put(2 * cb + 1, avg2<T, EXACT>(e00, e01), avg4<T, EXACT>(e00, e10, e01, e11));
 }
 
 MgSmoothArgs smooth_args(const MgLevel &L, const void *f, const void *uin, void *uout, int k, double omega,
@@ -492,6 +579,10 @@ void launch_smooth(hj_handle *h, int l, int cur, int tx, int ty, int k, double o
     // warps a CTA before rows are added to a thread
     while (f64 && rpt > 1 && tx * (ty / rpt) < 128) rpt /= 2;
     const dim3 block(tx, ty / rpt), grid((L.nx + tx - 1) / tx, (L.ny + ty - 1) / ty);
+    if (!f64 && a.stage == MG_PLAIN && tx == 32 && ty % 4 == 0 && ty <= 32) {
+        mg_smooth_rows_kernel<<<grid, 32 * (ty / 4), 0, s>>>(a);
+        return;
+    }
     const int smem = 2 * (tx + 2) * (ty + 2) * (f64 ? 8 : 4);
 #define HJ_MG_SMOOTH(T, EX, ST)                                                            \
     do {                                                                                   \

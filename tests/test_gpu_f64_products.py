@@ -82,3 +82,27 @@ def test_products_at_the_edges_of_the_range(shape, asym, scale, zeros):
         got = _cycles(p, 2, tile_x=tx, tile_y=ty, tile_threads=th, k=5, fixed_cycles=3, pipeline=0)
         ref = oracle.run_fixed(p.st, p.f, p.u0, 3, tx, ty, 5)
         assert np.array_equal(got, ref), (tx, ty, th, rel_max(got, ref))
+
+
+@pytest.mark.parametrize("shape,tile,prec", [((191, 127), (32, 8), "f32"), ((191, 127), (32, 32), "f32"),
+                                              ((255, 31), (32, 4), "f32"), ((191, 95), (32, 32), "f64"),
+                                              ((127, 127), (1, 8), "f64")])
+def test_multigrid_transfer_and_smoothing_edges(shape, tile, prec):
+    """Ragged last subdomains of every level, levels of one CTA, and coarse levels
+    of one row: binary64 bitwise, binary32 within 1e-5 of the oracle's V-cycles."""
+    import torch
+    p = W.random_bc_problem(2, *shape, seed=21, sigma_kind="const", asym=True)
+    L = oracle.mg_max_levels(*shape)
+    dt = torch.float32 if prec == "f32" else torch.float64
+    s = gpu_solver(p, method="mg", precision=prec, tile_x=tile[0], tile_y=tile[1], k=3, mg_pre=2, mg_post=1, fixed_cycles=2)
+    u = to_dev(p.u0, 2, dt)
+    s.solve(to_dev(p.f, 2, dt), u)
+    s.close()
+    ref = p.u0
+    for _ in range(2):
+        ref = oracle.mg_vcycle(p.st, p.f, ref, L, 2, 1, tile[0], tile[1], 3, 0.8)
+    got = to_host(u, shape[0])
+    if prec == "f64":
+        assert np.array_equal(got, ref), rel_max(got, ref)
+    else:
+        assert rel_max(got, ref) <= 1e-5
