@@ -176,7 +176,8 @@ const TileKernelInfo *find_tile(int fam, int dim, int tx, int ty, int threads = 
 // subdomains) 6.21, -, 4.46; 512 x 512 (256) 6.37, 5.52, 5.90; with 8
 // overlapping points and k = 64 (484) 10.2, 10.8, 11.2.  Binary64 (its first
 // variant has four warps, one per sub-partition's FP64 pipe) gains the waits of
-// one warp filled by another: k = 16 with 2, 4, 8 warps: 256 x 256 63, 40, 36;
+// one warp filled by another (and clusters of CTAs below that, cluster_choice):
+// k = 16 with 2, 4, 8 warps: 256 x 256 63, 40, 36;
 // 500 x 300 (160) 87, 77, 75; 900 x 800 (725) 194, 177, 175; 3001 x 2003
 // (5,922) 1352, 1315, 1315.
 int default_threads(int fam, const hj_desc &d, const hj_params &p, int nsm) {
@@ -191,6 +192,22 @@ int default_threads(int fam, const hj_desc &d, const hj_params &p, int nsm) {
             best = std::max(best, k[i].threads);
     const TileKernelInfo *first = find_tile(fam, 2, p.tile_x, p.tile_y);
     return first && best > first->threads ? best : 0;
+}
+
+// Binary64 32 x 32 subdomains on a cluster of CTAs, where the caller leaves the
+// threads to the library and the grid has so few subdomains that every CTA finds
+// an SM of its own (measured beside hier2d_cluster_kernel); else null.
+const TileKernelInfo *cluster_choice(int fam, const hj_desc &d, const hj_params &p, int nsm) {
+    if (fam != FAM_F64 || d.dim != 2 || p.method != HJ_METHOD_HIER || d.coef || p.persistent == 1 || p.pipeline == 1 ||
+        p.tile_threads || p.tile_x != 32 || p.tile_y != 32)
+        return nullptr;
+    const long long n = (long long)subdomain_count(d.nx, p.tile_x, p.overlap_x) *
+                        subdomain_count(d.ny, p.tile_y, p.overlap_y);
+    int cnt = 0;
+    const TileKernelInfo *k = cluster_kernels_f64(&cnt);
+    for (int i = 0; i < cnt; ++i)
+        if (n * k[i].cluster <= nsm) return &k[i];
+    return nullptr;
 }
 
 double now_ms() {
@@ -280,6 +297,7 @@ void geometry(const hj_handle *h, const TileKernelInfo *ki, bool classic, dim3 *
     if (h->d.dim == 2) {
         *grid = ovl ? dim3(subdomain_count(nx, ki->tx, h->p.overlap_x), subdomain_count(ny, ki->ty, h->p.overlap_y))
                     : dim3((nx + ki->tx - 1) / ki->tx, (ny + ki->ty - 1) / ki->ty);
+        grid->x *= ki->cluster;
     } else {
         const int tiles = ovl ? subdomain_count(nx, ki->tx, h->p.overlap_x) : (nx + ki->tx - 1) / ki->tx;
         *grid = dim3((tiles + ki->tiles_per_cta - 1) / ki->tiles_per_cta, ny);
@@ -603,7 +621,8 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
             if (!b2) return seterr(HJ_ERR_CUDA, "internal: deferred residual runs need a third iterate buffer");
             // (the reduction workspace holds two slots of one partial per subdomain)
             const long long nb = (long long)pl->grid.x * pl->grid.y;
-            pl->grid = dim3((unsigned)nb + 1);   // CTA 0 folds, CTA 1 + t sweeps subdomain t
+            // CTA (cluster) 0 folds, CTA (cluster) 1 + t sweeps subdomain t
+            pl->grid = dim3((unsigned)nb + ki->cluster);
             CKS(ensure_reduction(h, (size_t)nb));
             void *bufs[3] = {b0, b1, b2};
             pl->deferred = true;
@@ -1108,7 +1127,7 @@ void fill_stats_config(const hj_handle *h, hj_stats *st, double t0) {
     st->tile_y = h->d.dim == 2 ? h->p.tile_y : 1;
     st->k = h->p.k;
     const TileKernelInfo *tk = h->ir ? h->k_inner : h->k_outer;
-    st->tile_threads = tk            ? tk->threads / tk->tiles_per_cta
+    st->tile_threads = tk            ? tk->threads * tk->cluster / tk->tiles_per_cta
                        : vc_rows(h) ? 8 * h->p.tile_y
                           : (h->d.coef || h->p.method == HJ_METHOD_MG) ? h->p.tile_x * (h->d.dim == 2 ? h->p.tile_y : 1)
                           : h->k3                                      ? 32
@@ -1475,7 +1494,8 @@ int hj_create(hj_handle **out, const hj_desc *desc, const hj_params *params) {
         // (variable coefficients run their own thread-per-point kernel: any
         // subdomain of at most 1024 points)
         const int th = p.tile_threads ? p.tile_threads : default_threads(h->fam_outer, d, p, h->nsm);
-        h->k_outer = d.coef ? nullptr : find_tile(h->fam_outer, d.dim, p.tile_x, p.tile_y, th);
+        h->k_outer = d.coef ? nullptr : cluster_choice(h->fam_outer, d, p, h->nsm);
+        if (!h->k_outer && !d.coef) h->k_outer = find_tile(h->fam_outer, d.dim, p.tile_x, p.tile_y, th);
         if (!h->k_outer && !d.coef)
             HJ_FAIL(HJ_ERR_UNSUPPORTED, "tile %dx%d (%d threads) not built for this precision", p.tile_x, p.tile_y,
                     p.tile_threads);
@@ -1495,6 +1515,11 @@ int hj_create(hj_handle **out, const hj_desc *desc, const hj_params *params) {
             geometry(h, &k[i], false, &g, &b);
             maxb = std::max(maxb, (size_t)g.x * g.y);
         }
+    }
+    if (h->k_outer) {
+        dim3 g, b;
+        geometry(h, h->k_outer, false, &g, &b);
+        maxb = std::max(maxb, (size_t)g.x * g.y);
     }
     if (d.dim == 3) {
         const long long gx = (d.nx + 31) / 32, gy = (d.ny + 7) / 8;

@@ -571,7 +571,32 @@ __device__ __forceinline__ float sweeps2d_fold(Tile2D<float, C, R, SIG> &t, cons
     return acc;
 }
 
-template <typename T, int C, int R, int NW, int H, bool EXACT, bool SIG, bool RES, bool PART, bool OVL = false>
+// Cluster barrier (all threads of the cluster's CTAs), and a store into the
+// shared memory of another CTA of the cluster at this CTA's address p.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ unsigned remote_addr(const void *p, unsigned rank) {
+    unsigned r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_remote(const double *p, unsigned rank, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote_addr(p, rank)), "d"(v) : "memory");
+}
+__device__ __forceinline__ void st_remote(const int *p, unsigned rank, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(remote_addr(p, rank)), "r"(v) : "memory");
+}
+
+// CL > 1: the subdomain's NW warps are spread over the CL CTAs of a cluster, NW / CL
+// consecutive warps each; an edge row that a neighbouring CTA reads is stored into
+// that CTA's exchange buffer, and the barrier is the cluster's.
+template <typename T, int C, int R, int NW, int H, bool EXACT, bool SIG, bool RES, bool PART, bool OVL = false, int CL = 1>
 __device__ __forceinline__ typename std::conditional<EXACT, double, T>::type
 sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, const int yb, const int nx,
          const int ny, T *xbuf, const Own own = Own{0, 0, 0, 0}, DbgWord *dbg = nullptr) {
@@ -582,7 +607,9 @@ sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, 
     if constexpr (PACK) {
         return sweeps2d_fold<C, R, NW, H, SIG, RES, OVL>(t, kc, k, x0, yb, xbuf, own, dbg);
     } else {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int NWC = NW / CL;   // warps of this CTA
+    const unsigned rank = CL > 1 ? cluster_rank() : 0u;
+    const int lane = threadIdx.x & 31, w = (int)(threadIdx.x >> 5) + (CL > 1 ? (int)rank * NWC : 0);
     const int li = lane % L, hb = lane / L;
     const int xl = x0 + li * C;
     const unsigned m_first = lane_mask(li == 0), m_last = lane_mask(li == L - 1);   // halo lanes of a row
@@ -779,8 +806,14 @@ sweeps2d(Tile2D<T, C, R, SIG> &t, const Coef<T> &kc, const int k, const int x0, 
                 const int i0 = (w * 2 + 0) * TX + li * C + c, i1 = (w * 2 + 1) * TX + li * C + c;
                 if (hb == 0 && HJ_IN(dbg, o + i0, NX, 16)) buf[i0] = first[c];
                 if (hb == H - 1 && HJ_IN(dbg, o + i1, NX, 16)) buf[i1] = last[c];
+                if constexpr (CL > 1) {
+                    const int wc = (int)(threadIdx.x >> 5);
+                    if (wc == 0 && rank > 0 && HJ_IN(dbg, o + i0, NX, 16)) st_remote(buf + i0, rank - 1, first[c]);
+                    if (wc == NWC - 1 && rank < CL - 1 && HJ_IN(dbg, o + i1, NX, 16)) st_remote(buf + i1, rank + 1, last[c]);
+                }
             }
-            __syncthreads();
+            if constexpr (CL > 1) cluster_sync();
+            else __syncthreads();
             if (w > 0 && hb == 0) {
 #pragma unroll
                 for (int c = 0; c < C; ++c) {
@@ -931,6 +964,78 @@ __global__ void __launch_bounds__(32 * NW) hier2d_kernel(const CycArgs a) {
         // answer stands, and the next solve resets the control block)
         if (a.part_w) write_cta_partial<NW>(a.part_w + tile, acc);
         else if (!stop) reduce_grid_acc(a.red, acc);
+    }
+}
+
+// Binary64 subdomain on a cluster of CL CTAs, for grids with few subdomains.  A
+// binary64 cycle of such a grid is the FP64 pipes of the SMs its subdomains sit on
+// while the others idle; spread over CL SMs, a 32 x 32 subdomain's rows are two to a
+// warp (NWC warps a CTA, NWC CL R = 32), and the edge rows between CTAs travel
+// through distributed shared memory.  Same values as hier2d_kernel, bit for bit.
+// Runs where CL CTAs per subdomain leave at most one CTA on an SM.  Measured, us a
+// cycle, against eight warps on one SM: 36 subdomains or fewer (four CTAs each)
+// k = 16 33 -> 18, k = 4 9.7 -> 6.1, k = 1 4.5 -> 3.2; 256 x 256 (64, two CTAs each)
+// k = 16 33 -> 24.5, k = 4 9.7 -> 8.2, k = 1 4.5 -> 3.9.  What is left of a
+// subiteration is the cluster's barrier and the stores between its SMs.
+// Deferred fold as in hier2d_kernel (cluster 0 folds: its CTA 0); one partial per CTA.
+template <int NWC, int CL, bool SIG, bool RES, bool OVL>
+__global__ void __launch_bounds__(32 * NWC) __cluster_dims__(CL, 1, 1) hier2d_cluster_kernel(const CycArgs a) {
+    constexpr int NW = NWC * CL, TX = 32, TY = 32, R = TY / NW;
+    static_assert(R >= 2 && NW * R == TY, "whole rows");
+    const unsigned rank = cluster_rank();
+    int bx = (int)blockIdx.x / CL, by = blockIdx.y, part = 0;
+    __shared__ int s_stop;
+    __shared__ double xbuf[2 * NW * 2 * TX];
+    if constexpr (RES) {
+        if (a.part_w) {
+            if (bx == 0) {
+                if (rank == 0 && ((volatile Ctl *)a.red.ctl)->done < 0)
+                    deferred_fold_parts<NWC>(a.red, a.part_r, (int)gridDim.x - CL, a.parity);
+                return;
+            }
+            const int tile = bx - 1;
+            part = (int)blockIdx.x - CL;
+            by = tile / a.jx;
+            bx = tile - by * a.jx;
+        }
+        cluster_sync();   // every CTA of the cluster has started: its shared memory can be written
+        // one answer for the whole cluster: the fold of this launch may be setting the flag now
+        if (rank == 0 && threadIdx.x < CL) {
+            volatile Ctl *ctl = a.red.ctl;
+            const int stop = (ctl->done >= 0) | (a.part_w ? ctl->fold_only[a.parity] : 0);
+            st_remote(&s_stop, threadIdx.x, __shfl_sync((1u << CL) - 1u, stop, 0));
+        }
+    }
+    int x0 = 1 + bx * TX, y0 = 1 + by * TY;
+    Own own{0, 0, 0, 0};
+    if constexpr (OVL) {
+        const Span sx = subdomain_span(bx, a.jx, a.nx, TX, a.ox);
+        const Span sy = subdomain_span(by, a.jy, a.ny, TY, a.oy);
+        x0 = sx.start;
+        y0 = sy.start;
+        own = Own{sx.lo, sx.hi, sy.lo, sy.hi};
+    }
+    const int yb = y0 + ((int)rank * NWC + (int)(threadIdx.x >> 5)) * R;
+    const Coef<double> kc = make_coef<double>(a);
+    double acc = 0.0;
+    auto body = [&](auto part_tag) {
+        constexpr bool PART = decltype(part_tag)::value;
+        Tile2D<double, 1, R, SIG> t;
+        stage2d_global<double, double, 1, R, 1, true, SIG, PART>(t, a, kc, x0, yb);
+        // every CTA of the cluster has started (its exchange buffer can be written), and s_stop
+        // is there; no CTA leaves before the last such barrier, so none is written after it left
+        cluster_sync();
+        if constexpr (RES) {
+            if (s_stop) return;
+        }
+        acc = sweeps2d<double, 1, R, NW, 1, true, SIG, RES, PART, OVL, CL>(t, kc, a.k, x0, yb, a.nx, a.ny, xbuf, own, a.dbg);
+        store2d<double, double, 1, R, 1, SIG, PART, OVL>(t, a, x0, yb, own);
+    };
+    if (x0 + TX - 1 <= a.nx && y0 + TY - 1 <= a.ny) body(std::integral_constant<bool, false>());
+    else body(std::integral_constant<bool, true>());
+    if constexpr (RES) {
+        if (a.part_w) write_cta_partial<NWC>(a.part_w + part, acc);
+        else if (!s_stop) reduce_grid_acc(a.red, acc);
     }
 }
 
@@ -1514,6 +1619,14 @@ __global__ void __launch_bounds__(256) classic1d_kernel(const CycArgs a) {
        hj::hier2d_kernel<S, T, C, R, NW, H, EX, false, true, true>},                                  \
       {hj::hier2d_kernel<S, T, C, R, NW, H, EX, true, false, true>,                                   \
        hj::hier2d_kernel<S, T, C, R, NW, H, EX, true, true, true>}}}
+// 32 x 32 binary64 on a cluster: threads are the CTA's, cluster its CTAs per subdomain
+#define HJ_K2DCL(NWC, CL)                                                                             \
+    {2, 32, 32, 32 * (NWC), 1,                                                                       \
+     {{hj::hier2d_cluster_kernel<NWC, CL, false, false, false>, hj::hier2d_cluster_kernel<NWC, CL, false, true, false>}, \
+      {hj::hier2d_cluster_kernel<NWC, CL, true, false, false>, hj::hier2d_cluster_kernel<NWC, CL, true, true, false>}},  \
+     {{hj::hier2d_cluster_kernel<NWC, CL, false, false, true>, hj::hier2d_cluster_kernel<NWC, CL, false, true, true>},   \
+      {hj::hier2d_cluster_kernel<NWC, CL, true, false, true>, hj::hier2d_cluster_kernel<NWC, CL, true, true, true>}},    \
+     (CL)}
 #define HJ_K1D(S, T, C, WPT, WPB, EX)                                                                \
     {1, 32 * (C) * (WPT), 1, 32 * (WPT) * (WPB), (WPB),                                              \
      {{hj::hier1d_kernel<S, T, C, WPT, WPB, EX, false, false>,                                       \

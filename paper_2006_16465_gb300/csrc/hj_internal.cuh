@@ -440,6 +440,7 @@ struct TileKernelInfo {
     int tiles_per_cta;  // 1D packs several tiles per CTA
     CycKernel fn[2][2]; // [sig][res]
     CycKernel ovl[2][2];// [sig][res] overlapping subdomains (null for classic kernels)
+    int cluster = 1;    // CTAs per subdomain (a cluster along x)
 };
 
 // Variable-coefficient kernels: [dim - 1][res], one thread per point, dynamic
@@ -478,6 +479,8 @@ int aux_max_blocks3(int nx, int ny, int nz);
 enum KernelFamily { FAM_F64 = 0, FAM_F32 = 1, FAM_BF16 = 2 };
 const TileKernelInfo *tile_kernels_f64(int *n);
 const TileKernelInfo *tile_kernels_f32(int *n);
+// binary64 32 x 32 subdomains on clusters, widest first (not listed as variants)
+const TileKernelInfo *cluster_kernels_f64(int *n);
 const TileKernelInfo *tile_kernels_bf16(int *n);
 const TileKernelInfo *classic_kernels_f64(int *n);
 const TileKernelInfo *classic_kernels_f32(int *n);

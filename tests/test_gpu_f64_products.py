@@ -106,3 +106,23 @@ def test_multigrid_transfer_and_smoothing_edges(shape, tile, prec):
         assert np.array_equal(got, ref), rel_max(got, ref)
     else:
         assert rel_max(got, ref) <= 1e-5
+
+
+@pytest.mark.parametrize("shape,sigma,asym,ovl,k", [((96, 70), "field", True, 0, 4), ((64, 64), "none", False, 0, 1),
+                                                     ((200, 150), "const", False, 0, 3), ((200, 150), "field", False, 6, 5),
+                                                     ((33, 250), "none", True, 0, 16), ((7, 5), "none", False, 0, 2)])
+def test_clusters_match_oracle(shape, sigma, asym, ovl, k):
+    """Few 32 x 32 subdomains: each runs on a cluster of CTAs (fixed cycles, and a
+    converging solve with the deferred fold); same iterates and stopping cycle."""
+    import torch
+    p = W.random_bc_problem(2, *shape, seed=13, sigma_kind=sigma, asym=asym)
+    kw = dict(tile_x=32, tile_y=32, k=k, overlap_x=min(ovl, 31), overlap_y=min(ovl, 31))
+    got = _cycles(p, 2, fixed_cycles=5, **kw)
+    assert np.array_equal(got, oracle.run_fixed(p.st, p.f, p.u0, 5, 32, 32, k, overlap=(ovl, ovl)))
+    s = gpu_solver(p, precision="f64", tol=1e-2, max_cycles=2000, check_every=8, **kw)
+    u = to_dev(p.u0, 2, torch.float64)
+    out = s.solve(to_dev(p.f, 2, torch.float64), u, check=False)
+    assert out["tile_threads"] == 512
+    s.close()
+    uo, c, status, _ = oracle.solve(p.st, p.f, p.u0, 1e-2, 2000, 32, 32, k, overlap=(ovl, ovl))
+    assert out["cycles"] == c and np.array_equal(to_host(u, shape[0]), uo)
