@@ -155,7 +155,8 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
     const size_t o_third = al(o_maps + (tma ? nprob * sizeof(PersistMaps) : 0));
     const size_t o_qprobs = al(o_third + (late ? nprob * sizeof(void *) : 0));
     const size_t o_qent = al(o_qprobs + (late ? nprob * sizeof(int) : 0));
-    const size_t total = al(o_qent + (late ? nitems * sizeof(int4) : 0));
+    const size_t o_sm = al(o_qent + (late ? nitems * sizeof(int4) : 0));
+    const size_t total = al(o_sm + (late ? kSmSlots * sizeof(int) : 0));
     CKS(ensure_scratch(h, total));
     unsigned char *hb = h->h_pstage;
     unsigned char *db = (unsigned char *)h->pscratch;
@@ -181,6 +182,7 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
     if (late)
         for (int p = 0; p < nprob; ++p) ((void **)(hb + o_third))[p] = probs[p].third;
     memset(hb + o_q + 4 * sizeof(int), 0, 2 * sizeof(long long) + sizeof(int4));
+    if (late) memset(hb + o_sm, 0, kSmSlots * sizeof(int));
     unsigned *hbar = (unsigned *)(hb + o_bar);
     hbar[0] = hbar[1] = 0u;
     ((int *)hbar)[2] = nprob;   // active
@@ -224,6 +226,7 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
     P.q_ent = late ? (int4 *)(db + o_qent) : nullptr;
     P.q_probs = late ? (int *)(db + o_qprobs) : nullptr;
     P.third = late ? (void *const *)(db + o_third) : nullptr;
+    P.sm_ctas = late ? (int *)(db + o_sm) : nullptr;
     int cap = 0, threads = 256;
     if (classic) {
         int occ = 0;
@@ -235,6 +238,11 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
     }
     if (cap < 1) return seterr(HJ_ERR_UNSUPPORTED, "persistent kernel does not fit on an SM");
     // (late: the checks of the cycle before are queue entries too)
+    // one-warp CTAs: two per scheduler.  At the full twelve per SM their copies, all
+    // issued behind the same barrier, wait 18 us for the first box; ten leave the
+    // schedulers uneven (64 problems of sides 64 to 512, all active: 12, 10, 8, 7, 6
+    // CTAs per SM 41.0, 41.1, 37.1, 38.9, 41.7 us a cycle)
+    if (late && !sig && threads == 32) cap = std::min(cap, 8 * h->nsm);
     L->grid = (int)std::min<long long>(nitems + (late ? nprob : 0), cap);
     L->threads = threads;
     L->smem = tma ? ki->tma_smem[sig] : 0;
@@ -326,6 +334,7 @@ struct BatchArgs {
     ProbState *state;         // the inner engine's per-problem state
     int *inner_active;        // the inner engine's count of active problems
     int *q_changed;           // the inner engine's queue: rebuild at the next launch
+    int *sm_ctas;             // its per-SM counters (nullable): zeroed for the next launch
     const int *aux_prob;      // per aux item: its problem
     double *aux_part;         // per aux item: its share of ||r||^2
     int *count;               // problems still refining (read by the host)
@@ -453,6 +462,7 @@ __global__ void __launch_bounds__(1024) batch_finalize_kernel(const BatchArgs A)
             mine += o.active;
         }
     }
+    if (A.sm_ctas && threadIdx.x < kSmSlots) A.sm_ctas[threadIdx.x] = 0;
     __shared__ int s_n[32];
     mine = __reduce_add_sync(0xffffffffu, mine);
     if (lane == 0) s_n[w] = mine;
@@ -711,6 +721,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
     B.state = L.P.state;
     B.inner_active = L.P.active;
     B.q_changed = L.P.q_changed;
+    B.sm_ctas = L.P.sm_ctas;
     B.aux_prob = (const int *)(dm + m_auxp);
     B.aux_part = (double *)(dm + m_part);
     B.count = (int *)(dm + m_word);

@@ -42,6 +42,8 @@ struct ProbState {
 
 struct PersistMaps;   // hj_persist_tma.cuh: per-problem tensor maps
 
+constexpr int kSmSlots = 512;   // counters of CTAs per SM (SM numbers beyond share them)
+
 struct PersistArgs {
     const CycArgs *probs;    // per problem: f, b0 (=uin), b1 (=uout), dinv, geometry, k, coefficients,
                              // red.tol, red.max_cycles, red.scale
@@ -74,6 +76,7 @@ struct PersistArgs {
     int *q_probs;            // [nprob] the active problems
     int4 *q_state;           // {entries in q_ent, active problems, CTAs of the next cycle, number of rebuilds}
     void *const *third;      // per problem: the third iterate buffer
+    int *sm_ctas;            // [kSmSlots] CTAs of the launch per SM (zero before it)
     // per-cycle log (nullable): [2 * n] = end time (ns), [2 * n + 1] = active points of the next cycle
     unsigned long long *tlog;
     long long *tlog_n;
@@ -236,13 +239,14 @@ __device__ __forceinline__ double cta_sum(A acc) {
     return s;
 }
 
-// Phase B for problem p (run by warp 0 of one CTA).
-__device__ __forceinline__ void retire_check(const PersistArgs &P, int p, int parity) {
+// Phase B for problem p (run by warp 0 of one CTA).  Lane 0 gets whether p retired.
+__device__ __forceinline__ int retire_check(const PersistArgs &P, int p, int parity) {
     const int lane = threadIdx.x & 31;
     const int i0 = P.prob_item0[p], n = P.prob_nitems[p];
     double s = 0.0;
     for (int i = lane; i < n; i += 32) s += __ldcg(&P.partial[(size_t)parity * P.nitems + i0 + i]);
     s = warp_sum(s);
+    int retire = 0;
     if (lane == 0) {
         volatile ProbState *st = P.state + p;
         const RedArgs &r = P.probs[p].red;
@@ -252,7 +256,7 @@ __device__ __forceinline__ void retire_check(const PersistArgs &P, int p, int pa
         const double first = st->res2_0;
         if (c == 0) st->res2_0 = res2;
         st->res2_last = res2;
-        int retire = 1;
+        retire = 1;
         if (!finite_bits(res2)) {
             st->status = HJ_ERR_DIVERGED;
             st->done = (int)c;
@@ -272,6 +276,7 @@ __device__ __forceinline__ void retire_check(const PersistArgs &P, int p, int pa
             if (P.q_changed) *(volatile int *)P.q_changed = 1;
         }
     }
+    return retire;
 }
 
 template <typename S, typename T, int C, int R, int NW, int H, bool EXACT, bool SIG>

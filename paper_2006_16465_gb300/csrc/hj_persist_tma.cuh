@@ -140,11 +140,16 @@ __global__ void __launch_bounds__(32 * NW) persist2d_tma_one_kernel(const Persis
 //   * the queue only shrinks within a launch, so a CTA whose number lies beyond
 //     its entries leaves for good, and the barrier counts those that stay;
 //   * barrier words are read and written with acquire and release instead of
-//     full fences.
+//     full fences;
+//   * CTAs are numbered breadth-first over the SMs (cta_rank): by block index the
+//     first 48 of a full launch sit on four SMs, twelve each, so that a queue of a
+//     few hundred entries swept at the speed of those four (15.5 us a cycle; 8 to 9
+//     with the numbering).
 // The residual sums, and with them every decision and iterate, are those of the
 // two-barrier kernel.  Measured (32 x 32, k = 32, binary32 inner cycles): 64
-// problems of sides 64 to 512 to 1e-8 1.13 -> 0.65 s; 8 sigma-field problems of
-// 256 x 256 to 1e-10, forward and adjoint, 0.41 -> 0.16 s.
+// problems of sides 64 to 512 to 1e-8 1.13 -> 0.55 s (0.65 with CTAs numbered by
+// block index, twelve per SM); 8 sigma-field problems of 256 x 256 to 1e-10, forward
+// and adjoint, 0.41 -> 0.16 s.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned *p, unsigned v) {
     unsigned r;
@@ -200,22 +205,32 @@ __device__ __forceinline__ void batch_queue_rebuild(const PersistArgs &P) {
     }
 }
 
-// Grid barrier over the `alive` CTAs of the cycle.  head receives the queue's
-// state for the next one.  False if the wait expired or a CTA recorded an error.
-__device__ __forceinline__ bool batch_barrier(const PersistArgs &P, int alive, unsigned &gen, int4 &head) {
-    __shared__ int s_last, s_ok;
+// Grid barrier over the `alive` CTAs of the cycle.  Nothing is read in it that the
+// two words do not carry: an arrival adds 1, and 2^16 if the CTA retired a problem,
+// so the last to arrive knows whether to rebuild the queue; the release word's
+// lowest bit tells the others whether it was rebuilt, and only then do they read
+// its state into head.  False if the wait expired or a CTA recorded an error.
+__device__ __forceinline__ bool batch_barrier(const PersistArgs &P, int alive, int retired, unsigned &word, int4 &head) {
+    __shared__ int s_last, s_state;
     __shared__ int4 s_head;
     __syncthreads();   // the CTA's stores are done
-    if (threadIdx.x == 0) s_last = atom_add_acq_rel(P.bar, 1u) == (unsigned)alive - 1u;
+    if (threadIdx.x == 0) {
+        const unsigned mine = 1u + (retired ? 0x10000u : 0u);
+        const unsigned now = atom_add_acq_rel(P.bar, mine) + mine;
+        s_last = (now & 0xffffu) == (unsigned)alive ? 1 + (now >= 0x10000u) : 0;
+    }
     __syncthreads();
+    const unsigned next = ((word >> 1) + 1u) << 1;
+    unsigned seen = next;
     int ok = 1;
     if (s_last) {
-        // one answer for every thread before the rebuild clears the flag
-        const int changed = __syncthreads_or(threadIdx.x == 0 && *(volatile int *)P.q_changed);
-        if (changed) batch_queue_rebuild(P);
-        __syncthreads();
+        const int changed = s_last == 2;
+        if (changed) {
+            batch_queue_rebuild(P);
+            __syncthreads();
+        }
         if (threadIdx.x == 0) {
-            *P.q_head = __ldcg(&P.q_state->z);
+            *P.q_head = changed ? __ldcg(&P.q_state->z) : alive;
             if (P.tlog) {
                 const long long n = *P.tlog_n;
                 if (n < P.tlog_cap) {
@@ -225,11 +240,12 @@ __device__ __forceinline__ bool batch_barrier(const PersistArgs &P, int alive, u
                 *P.tlog_n = n + 1;
             }
             *(volatile unsigned *)P.bar = 0u;
-            st_release(P.bar + 1, gen + 1u);
+            seen = next | (unsigned)changed;
+            st_release(P.bar + 1, seen);
         }
     } else if (threadIdx.x == 0) {
         const unsigned long long t0 = global_ns();
-        for (unsigned polls = 0; ld_acquire(P.bar + 1) == gen; ++polls) {
+        for (unsigned polls = 0; (seen = ld_acquire(P.bar + 1)) == word; ++polls) {
             if ((polls & 15u) == 15u) {
                 if (*(volatile int *)P.err) { ok = 0; break; }
                 if (global_ns() - t0 > P.timeout_ns) {
@@ -242,13 +258,32 @@ __device__ __forceinline__ bool batch_barrier(const PersistArgs &P, int alive, u
         }
     }
     if (threadIdx.x == 0) {
-        s_head = __ldcg(P.q_state);
-        s_ok = ok && *(volatile int *)P.err == 0;
+        if (ok && (seen & 1u)) s_head = __ldcg(P.q_state);
+        s_state = ok ? 1 + (int)(seen & 1u) : 0;
     }
     __syncthreads();
-    ++gen;
-    head = s_head;
-    return s_ok != 0;
+    const int state = s_state;
+    word = next | (state == 2 ? 1u : 0u);
+    if (state == 2) head = s_head;
+    return state != 0;
+}
+
+// This CTA's number when the launch's CTAs are counted SM by SM, one of each in
+// turn: (its place on its SM, its SM) in lexicographic order.  slot: its place;
+// the per-SM counts are complete (a grid barrier lies between).  Whole CTA calls.
+__device__ __forceinline__ int cta_rank(const int *sm_ctas, int sm, int slot) {
+    __shared__ int s_rank;
+    if (threadIdx.x < 32) {
+        int r = 0;
+        for (int m = threadIdx.x; m < kSmSlots; m += 32) {
+            const int c = __ldcg(sm_ctas + m);
+            r += min(c, slot) + (m < sm && c > slot ? 1 : 0);
+        }
+        r = __reduce_add_sync(FULL, r);
+        if (threadIdx.x == 0) s_rank = r;
+    }
+    __syncthreads();
+    return s_rank;
 }
 
 // Four-warp kernels with a sigma field are held to three CTAs per SM (at most
@@ -277,16 +312,22 @@ __global__ void __launch_bounds__(32 * NW, (NW == 4 && SIG) ? 3 : 0) persist2d_b
     }
     __syncthreads();
     unsigned nwait = 0;   // copies waited for (mbarrier phase parity)
-    unsigned gen = *(volatile unsigned *)(P.bar + 1);   // (moves only once every CTA has arrived)
-    int4 head;
+    unsigned word = *(volatile unsigned *)(P.bar + 1);   // (moves only once every CTA has arrived)
+    int4 head = make_int4(0, 0, 0, 0);
+    __shared__ int s_slot;   // (every lane of a warp is on one SM, and so is its CTA)
+    unsigned sm;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+    sm %= kSmSlots;
+    if (tid == 0) s_slot = atomicAdd(P.sm_ctas + sm, 1);
     // the queue of the first cycle is built behind a barrier
-    if (!batch_barrier(P, (int)gridDim.x, gen, head)) return;
+    if (!batch_barrier(P, (int)gridDim.x, 1, word, head)) return;
+    const int me = cta_rank(P.sm_ctas, (int)sm, s_slot);
     int4 first = make_int4(0, 0, 0, 0);
     int first_of = head.w - 1;   // the rebuild `first` was read from
     // every active problem advances once per cycle: `it` is its cycle index
     for (long long it = 0; it < P.max_iters; ++it) {
         const int cnt = head.x, alive = head.z, total = cnt + (it > 0 ? head.y : 0);
-        if (head.y == 0 || (int)blockIdx.x >= alive) return;
+        if (head.y == 0 || me >= alive) return;
         const int parity = (int)(it & 1), bi = (int)(it % 3), bo = (int)((it + 1) % 3);
         auto issue = [&](const int4 &e) {
             const PersistMaps &m = P.maps[e.y];
@@ -295,7 +336,7 @@ __global__ void __launch_bounds__(32 * NW, (NW == 4 && SIG) ? 3 : 0) persist2d_b
             tma_load_2d(sf, &m.mf, bar, e.z * TX, e.w * TY + 1);
             if constexpr (SIG) tma_load_2d(sd, &m.md, bar, e.z * TX, e.w * TY + 1);
         };
-        int i = blockIdx.x;
+        int i = me;
         if (first_of != head.w) {
             if (i < cnt) first = __ldcg(P.q_ent + i);
             first_of = head.w;
@@ -371,10 +412,11 @@ __global__ void __launch_bounds__(32 * NW, (NW == 4 && SIG) ? 3 : 0) persist2d_b
             e = enext;
         }
         // entries [cnt, total): the active problems' checks of the cycle before
+        int retired = 0;
         if (tid < 32) {
             int next = __shfl_sync(FULL, nidx, 0);
             while (i < total) {
-                retire_check(P, __ldcg(P.q_probs + (i - cnt)), parity ^ 1);
+                retired |= retire_check(P, __ldcg(P.q_probs + (i - cnt)), parity ^ 1);
                 i = next;
                 if (next < total) {
                     if (tid == 0) next = atomicAdd(P.q_head, 1);
@@ -384,7 +426,7 @@ __global__ void __launch_bounds__(32 * NW, (NW == 4 && SIG) ? 3 : 0) persist2d_b
         }
         fence_proxy_async_global();   // this cycle's stores, before the next cycle's copies
         if ((int)blockIdx.x == P.skip_barrier_cta) return;
-        if (!batch_barrier(P, alive, gen, head)) return;
+        if (!batch_barrier(P, alive, retired, word, head)) return;
     }
 }
 
