@@ -732,11 +732,17 @@ int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, 
     ro->res2_c = -1.0;
     CycArgs base = base_in;
     base.err = &h->ctl->err;
-    *h->h_ctl_init = Ctl{-1, HJ_OK, 0, 0.0, 0.0, 0, 0, 0.0, 0, 0, {0, 0}};
-    CKR(cudaMemcpyAsync(h->ctl, h->h_ctl_init, sizeof(Ctl), cudaMemcpyHostToDevice, s));
+    auto init_ctl = [&]() -> int {
+        *h->h_ctl_init = Ctl{-1, HJ_OK, 0, 0.0, 0.0, 0, 0, 0.0, 0, 0, {0, 0}};
+        CKR(cudaMemcpyAsync(h->ctl, h->h_ctl_init, sizeof(Ctl), cudaMemcpyHostToDevice, s));
+        return HJ_OK;
+    };
     if (fixed > 0) {
         Plan pl;
         CKS(make_plan(h, ki, pi, fam, classic, sig, false, base, b0, b1, nullptr, &pl));
+        // only the pipelined kernels touch the control block here (the error word of
+        // their bounded waits): the others need neither its copies nor a wait for them
+        if (pl.ppc) CKS(init_ctl());
         const long long reps = fixed / M;
         if (reps > 0) {
             cudaGraphExec_t ex;
@@ -745,16 +751,19 @@ int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, 
         }
         for (long long c = reps * M; c < fixed; ++c) plan_launch(pl, c, s);
         CKR(cudaGetLastError());
-        CKR(cudaMemcpyAsync(h->h_ctl, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
-        CKR(cudaEventRecord(h->ev, s));
-        CKR(cudaEventSynchronize(h->ev));
-        if (h->h_ctl->err) return seterr(HJ_ERR_TIMEOUT, "a bounded device wait expired (tile pipeline)");
+        if (pl.ppc) {
+            CKR(cudaMemcpyAsync(h->h_ctl, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
+            CKR(cudaEventRecord(h->ev, s));
+            CKR(cudaEventSynchronize(h->ev));
+            if (h->h_ctl->err) return seterr(HJ_ERR_TIMEOUT, "a bounded device wait expired (tile pipeline)");
+        }
         ro->c = fixed;
         ro->status = HJ_OK;
         ro->launched = fixed;
         ro->buf = (fixed & 1) ? b1 : b0;
         return HJ_OK;
     }
+    CKS(init_ctl());
     {
         const long long sw = base.red.stall_window;
         base.red = red_args(h, RED_CYCLE, tol, max_cycles);
