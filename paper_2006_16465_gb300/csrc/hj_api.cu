@@ -615,10 +615,9 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
     if (!want_ppc(h, pi, classic)) {
         geometry(h, ki, classic, &pl->grid, &pl->block);
         pl->fn = (!classic && overlapped(h)) ? ki->ovl[sig][res] : ki->fn[sig][res];
-        if (res && defer_hier(h, ki, classic)) {
+        if (res && b2 && defer_hier(h, ki, classic)) {
             // deferred fold: launch c reads B[c % 3], writes B[(c+1) % 3] and
             // its per-CTA partials to slot c % 2, folded by launch c + 1
-            if (!b2) return seterr(HJ_ERR_CUDA, "internal: deferred residual runs need a third iterate buffer");
             // (the reduction workspace holds two slots of one partial per subdomain)
             const long long nb = (long long)pl->grid.x * pl->grid.y;
             // CTA (cluster) 0 folds, CTA (cluster) 1 + t sweeps subdomain t
@@ -788,15 +787,16 @@ int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, 
         b2 = third.alias;
     } else if (deferred_run(h, ki, pi, classic)) {
         if (!third.slot) return seterr(HJ_ERR_CUDA, "internal: no slot for the third iterate buffer");
-        if (!*third.slot) {
-            if (dmalloc(third.slot, third.bytes) != cudaSuccess) {
-                cudaGetLastError();
-                *third.slot = nullptr;
+        if (!*third.slot && dmalloc(third.slot, third.bytes) != cudaSuccess) {
+            cudaGetLastError();
+            *third.slot = nullptr;
+            // the one-CTA-per-subdomain kernels run without it (grid reduction at a launch's end)
+            if (want_ppc(h, pi, classic) || want_ppc3(h, classic))
                 return seterr(HJ_ERR_NO_MEMORY, "third iterate buffer (%zu bytes)", third.bytes);
-            }
         }
         b2 = *third.slot;
-        CKR(launch_copy_ring(h->d.dim, third.esz, b0, b2, nullptr, base.ld, base.ps, h->d.nx, h->d.ny, h->d.nz, s));
+        if (b2)
+            CKR(launch_copy_ring(h->d.dim, third.esz, b0, b2, nullptr, base.ld, base.ps, h->d.nx, h->d.ny, h->d.nz, s));
     }
     Plan pl;
     CKS(make_plan(h, ki, pi, fam, classic, sig, true, base, b0, b1, b2, &pl));
@@ -915,7 +915,9 @@ int iterate(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int
             // runs beside the sweeps (32 x 32, k = 32, binary32 cycles:
             // 512 x 512 10.1 against 6.4 us a cycle, 64 x 64 8.8 against 6.5; 1D
             // binary64, 512 points 12.3 against 10.2)
-            use = pclassic && blocks <= cap;
+            // (in-place runs stay: their array is one cycle past the checked one
+            // there, two with the deferred fold)
+            use = (pclassic || h->p.in_place) && blocks <= cap;
         }
     }
     if (used_persistent) *used_persistent = use ? 1 : 0;

@@ -267,7 +267,8 @@ int tune_launch(const hj_desc &d, hj_params *p) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const long long ntiles = (long long)((d.nx + p->tile_x - 1) / p->tile_x) * ((d.ny + p->tile_y - 1) / p->tile_y);
-    if (p->pipeline == -1 && ntiles < 8LL * nsm) return HJ_OK;
+    // (binary64 runs the pipelined kernel on request only)
+    if (p->pipeline == -1 && (ntiles < 8LL * nsm || prec == HJ_PREC_F64)) return HJ_OK;
     std::string key = make_key(d, p->precision, p->tol);
     {
         char extra[96];

@@ -131,6 +131,7 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
     // the kernel of many problems decides one cycle late, over three buffers
     bool late = tma;
     for (auto &p : probs) late = late && p.third;
+    if (nprob > 1 && !late) tma = false;   // without third buffers: plain staging, two barriers
     long long nitems = 0, max_iters = 1;
     for (auto &p : probs) {
         nitems += p.blocks;
@@ -249,7 +250,6 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
     // late decisions: one grid barrier per cycle for any number of problems;
     // else one for a single problem and two for several (reduce, then retire
     // and rebuild the work queue), which several TMA-staged ones never take
-    if (tma && !late && nprob > 1) return seterr(HJ_ERR_CUDA, "internal: several problems need third iterate buffers");
     L->late = late;
     L->fn = classic ? (const void *)classic
             : late ? (const void *)ki->tma_fn[sig]
@@ -578,7 +578,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
     bool sig_any = false;
     for (int i = 0; i < nprob; ++i) sig_any |= descs[i].sigma != nullptr;
     std::vector<BProb> P(nprob);
-    size_t arena = 0;
+    size_t arena = 0, thirds = 0;   // workspace, and the part of it that the third correction buffers take
     for (int i = 0; i < nprob; ++i) {
         if (!f[i] || !u[i] || ((uintptr_t)f[i] & 15) || ((uintptr_t)u[i] & 15))
             return seterr(HJ_ERR_INVALID_ARG, "problem %d: f/u NULL or not 16-byte aligned", i);
@@ -592,6 +592,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         arena += ((size_t)b.rows * b.d.ld * 8 + 255) / 256 * 256;    // u2
         arena += (b.nin * 4 + 255) / 256 * 256;                       // r32
         arena += 3 * ((b.nin * dsz + 255) / 256 * 256);               // dA, dB, dC
+        thirds += (b.nin * dsz + 255) / 256 * 256;
         if (sig_any) arena += (b.nin * 4 + 255) / 256 * 256;          // per-point 1/d (binary32)
     }
     if (arena > h->barena_bytes) {
@@ -600,8 +601,15 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         h->barena = nullptr;
         h->barena_bytes = 0;
         if (dmalloc(&h->barena, arena) != cudaSuccess) {
+            // without the third correction buffers the plain-staging engine runs
             cudaGetLastError();
-            return seterr(HJ_ERR_NO_MEMORY, "batched workspace of %zu bytes", arena);
+            arena -= thirds;
+            thirds = 0;
+            if (dmalloc(&h->barena, arena) != cudaSuccess) {
+                cudaGetLastError();
+                h->barena = nullptr;
+                return seterr(HJ_ERR_NO_MEMORY, "batched workspace of %zu bytes", arena);
+            }
         }
         h->barena_bytes = arena;
     }
@@ -611,7 +619,10 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         b.r32 = (float *)ap; ap += (b.nin * 4 + 255) / 256 * 256;
         b.dA = ap; ap += (b.nin * dsz + 255) / 256 * 256;
         b.dB = ap; ap += (b.nin * dsz + 255) / 256 * 256;
-        b.dC = ap; ap += (b.nin * dsz + 255) / 256 * 256;
+        b.dC = nullptr;
+        if (thirds) {
+            b.dC = ap; ap += (b.nin * dsz + 255) / 256 * 256;
+        }
         b.dinv = nullptr;
         if (sig_any) {
             b.dinv = (float *)ap; ap += (b.nin * 4 + 255) / 256 * 256;
@@ -623,7 +634,7 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         CKR(cudaMemsetAsync(b.r32, 0, b.nin * 4, s));
         CKR(cudaMemsetAsync(b.dA, 0, b.nin * dsz, s));
         CKR(cudaMemsetAsync(b.dB, 0, b.nin * dsz, s));
-        CKR(cudaMemsetAsync(b.dC, 0, b.nin * dsz, s));
+        if (b.dC) CKR(cudaMemsetAsync(b.dC, 0, b.nin * dsz, s));
     }
     // the inner engine over every problem of the batch (its work queue holds
     // the items of the problems still refining)
