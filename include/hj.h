@@ -185,11 +185,12 @@ typedef struct {
                              subdomain with cp.async; 0 = one warp per
                              subdomain; -1 = automatic: binary32 grids of at
                              least 8 subdomains per SM (subdomains at least 16
-                             wide) run the TMA-pipelined kernel (one warp per
+                             wide) run the TMA-pipelined kernel (one or two warps per
                              CTA walking subdomains), others one warp per
                              subdomain                                        */
     int tile_threads;     /* threads per subdomain (one warp per band of rows);
-                             0 = the default for the tile shape; the built
+                             0 = the default for the tile shape and the number
+                             of subdomains; the built
                              combinations are listed by hj_tile_variants()      */
     int pipeline_stages;  /* TMA-pipelined kernel: shared-memory stages per CTA
                              (binary32 / bfloat16: 1 or 2, binary64: 2; 0 = the

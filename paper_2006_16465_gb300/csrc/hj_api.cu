@@ -514,7 +514,7 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
         // seven-point extension: warp-per-subdomain register kernel, or the
         // classic thread-per-point sweep
         if (want_ppc3(h, classic)) {
-            // TMA-pipelined: one warp per CTA walks subdomains, the next one's
+            // TMA-pipelined: one or two warps per CTA walk subdomains, the next ones'
             // boxes copied in while the current one sweeps; residual folded by
             // the next launch over three rotating iterate buffers
             if (res && !b2) return seterr(HJ_ERR_CUDA, "internal: pipelined residual runs need a third iterate buffer");

@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(32 * NW, 3) hier3d_pk_kernel(const CycArgs a) 
 
 // ---------------------------------------------------------------------------
 // TMA-pipelined binary32 variant for grids much larger than the resident CTAs
-// (the 3D counterpart of ppc2d_kernel).  One warp per CTA walks a static list
+// (the 3D counterpart of ppc2d_kernel).  A CTA (NS warps, below) walks a static list
 // of subdomains (t = blockIdx.x + i gridDim.x, x fastest); one lane issues
 // cp.async.bulk.tensor copies of the next subdomain's iterate box (subdomain
 // + halo) and RHS box into shared memory, completing on an mbarrier, while
