@@ -372,7 +372,7 @@ __device__ __forceinline__ double corr(const DS *p) { return (double)(float)*p; 
 
 // INIT: r = f - A u[cur] for every problem; else u[cur ^ 1] = u[cur] + d and
 // r = f - A u[cur ^ 1] for the refining problems (d = the inner solve's last
-// buffer, by the parity of its cycle count).  r goes to r32 and each aux
+// buffer: its cycle count modulo the number of buffers it rotates through).  r goes to r32 and each aux
 // item's ||r||^2 share to aux_part (fixed order within the item).
 template <typename DS, bool INIT>
 __global__ void __launch_bounds__(256) batch_residual_kernel(const BatchArgs A) {
@@ -380,7 +380,10 @@ __global__ void __launch_bounds__(256) batch_residual_kernel(const BatchArgs A) 
     for (int a = blockIdx.x; a < A.naux; a += gridDim.x) {
         const int p = A.aux_prob[a];
         const BOuter o = A.outer[p];
-        if (!INIT && !o.active) continue;
+        const int done = INIT ? 0 : A.state[p].done;
+        // (done < 0: a wait of the inner launch expired, which the call reports;
+        // there is no correction to add, and the iterate stays)
+        if (!INIT && (!o.active || done < 0)) continue;
         const BDev b = A.prob[p];
         int i, j;
         double rr = 0.0;
@@ -393,7 +396,7 @@ __global__ void __launch_bounds__(256) batch_residual_kernel(const BatchArgs A) 
             const double *u = b.u[o.cur];
             double uc = u[q], uW = u[q - 1], uE = u[q + 1], uS = u[q - b.ld], uN = u[q + b.ld];
             if constexpr (!INIT) {
-                const DS *d = (const DS *)b.d[A.state[p].done % A.nbuf];
+                const DS *d = (const DS *)b.d[done % A.nbuf];
                 uc = __dadd_rn(uc, corr(d + q2));
                 uW = __dadd_rn(uW, corr(d + q2 - 1));
                 uE = __dadd_rn(uE, corr(d + q2 + 1));
@@ -432,7 +435,7 @@ __global__ void __launch_bounds__(1024) batch_finalize_kernel(const BatchArgs A)
     int mine = 0;
     for (int p = w; p < A.nprob; p += nw) {
         BOuter o = A.outer[p];
-        if (o.active) {
+        if (o.active && (INIT || A.state[p].done >= 0)) {   // (done < 0: batch_residual_kernel left it as it was)
             const BDev &b = A.prob[p];
             double s = 0.0;
             for (int k = lane; k < b.naux; k += 32) s += A.aux_part[b.aux0 + k];
