@@ -515,7 +515,16 @@ CycArgs prob_args(const hj_desc &d, const hj_params &p, bool transpose = false) 
     return a;
 }
 
-int validate_desc(const hj_desc &d, int i) {
+// Smallest per-point screening of a sigma array, read once per distinct array and
+// size of one call (a later call may find other values at the same address).
+struct SigmaMin {
+    const double *sigma;
+    int nx, ny;
+    long long ld;
+    double m;
+};
+
+int validate_desc(const hj_desc &d, int i, std::vector<SigmaMin> &seen, cudaStream_t s) {
     if (d.dim != 2) return seterr(HJ_ERR_INVALID_ARG, "problem %d: batched solves are 2D", i);
     if (d.nx < 1 || d.ny < 1 || d.ny > 524280) return seterr(HJ_ERR_INVALID_ARG, "problem %d: bad size", i);
     if (d.dtype != HJ_F64) return seterr(HJ_ERR_INVALID_ARG, "problem %d: batched solves take binary64 arrays", i);
@@ -525,20 +534,24 @@ int validate_desc(const hj_desc &d, int i) {
     const double off = fabs(d.cW) + fabs(d.cE) + fabs(d.cS) + fabs(d.cN);
     double dd = d.cD + d.sigma_const;
     if (d.sigma) {
-        // smallest per-point screening (read once per distinct sigma array)
-        static thread_local const double *last = nullptr;
-        static thread_local double last_min = 0.0;
-        if (d.sigma != last) {
+        auto it = std::find_if(seen.begin(), seen.end(), [&](const SigmaMin &e) {
+            return e.sigma == d.sigma && e.nx == d.nx && e.ny == d.ny && e.ld == d.ld;
+        });
+        if (it == seen.end()) {
+            // (on the call's stream: behind the work that writes sigma)
             std::vector<double> hs((size_t)(d.ny + 2) * d.ld);
-            if (cudaMemcpy(hs.data(), d.sigma, hs.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
+            if (cudaMemcpyAsync(hs.data(), d.sigma, hs.size() * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                cudaStreamSynchronize(s) != cudaSuccess) {
+                cudaGetLastError();
                 return seterr(HJ_ERR_CUDA, "problem %d: reading sigma", i);
+            }
             double m = INFINITY;
             for (int j = 1; j <= d.ny; ++j)
                 for (int x = 1; x <= d.nx; ++x) m = std::min(m, hs[(size_t)j * d.ld + x]);
-            last = d.sigma;
-            last_min = m;
+            seen.push_back(SigmaMin{d.sigma, d.nx, d.ny, d.ld, m});
+            it = seen.end() - 1;
         }
-        dd += last_min;
+        dd += it->m;
     }
     if (!(dd > 0.0) || dd < off) return seterr(HJ_ERR_NOT_DIAG_DOMINANT, "problem %d: not diagonally dominant", i);
     return HJ_OK;
@@ -560,7 +573,8 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
     cudaStream_t s = (cudaStream_t)stream;
     hj_params par = h->p;
     const int fam = h->fam_inner;
-    for (int i = 0; i < nprob; ++i) CKS(validate_desc(descs[i], i));
+    std::vector<SigmaMin> sigmas;
+    for (int i = 0; i < nprob; ++i) CKS(validate_desc(descs[i], i, sigmas, s));
     // autotune: one tile variant for the launch and k per size class (largest
     // side up to 128, 256, 384, beyond), by the batched cost model
     std::vector<int> kprob(nprob, par.k);
