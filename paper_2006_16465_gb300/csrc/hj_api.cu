@@ -179,9 +179,10 @@ const TileKernelInfo *find_tile(int fam, int dim, int tx, int ty, int threads = 
 // one warp filled by another (and clusters of CTAs below that, cluster_choice):
 // k = 16 with 2, 4, 8 warps: 256 x 256 63, 40, 36;
 // 500 x 300 (160) 87, 77, 75; 900 x 800 (725) 194, 177, 175; 3001 x 2003
-// (5,922) 1352, 1315, 1315.
+// (5,922) 1352, 1315, 1315.  In-place runs choose for the persistent engine instead
+// (in_place_threads).
 int default_threads(int fam, const hj_desc &d, const hj_params &p, int nsm) {
-    if (d.dim != 2 || p.method != HJ_METHOD_HIER || d.coef || p.persistent == 1 || p.pipeline == 1) return 0;
+    if (d.dim != 2 || p.method != HJ_METHOD_HIER || d.coef || p.persistent == 1 || p.pipeline == 1 || p.in_place) return 0;
     const long long n = (long long)subdomain_count(d.nx, p.tile_x, p.overlap_x) *
                         subdomain_count(d.ny, p.tile_y, p.overlap_y);
     const int want = fam == FAM_F64 ? (n <= 2LL * nsm ? 256 : 0) : n <= nsm ? 128 : n <= 2LL * nsm ? 64 : 0;
@@ -199,7 +200,7 @@ int default_threads(int fam, const hj_desc &d, const hj_params &p, int nsm) {
 // an SM of its own (measured beside hier2d_cluster_kernel); else null.
 const TileKernelInfo *cluster_choice(int fam, const hj_desc &d, const hj_params &p, int nsm) {
     if (fam != FAM_F64 || d.dim != 2 || p.method != HJ_METHOD_HIER || d.coef || p.persistent == 1 || p.pipeline == 1 ||
-        p.tile_threads || p.tile_x != 32 || p.tile_y != 32)
+        p.in_place || p.tile_threads || p.tile_x != 32 || p.tile_y != 32)
         return nullptr;
     const long long n = (long long)subdomain_count(d.nx, p.tile_x, p.overlap_x) *
                         subdomain_count(d.ny, p.tile_y, p.overlap_y);
@@ -305,6 +306,31 @@ void geometry(const hj_handle *h, const TileKernelInfo *ki, bool classic, dim3 *
     *block = dim3(ki->threads);
 }
 
+// Threads per subdomain of an in-place 2D run where the caller leaves the choice:
+// the first variant whose persistent kernel holds the whole grid (iterate runs it:
+// binary64 32 x 32, four warps up to three or four CTAs an SM, then two); 0 if none
+// does.
+int in_place_threads(hj_handle *h, int fam, bool sig, int *threads) {
+    *threads = 0;
+    if (!h->p.in_place || h->d.dim != 2 || h->p.method != HJ_METHOD_HIER || h->p.persistent != -1 || h->d.coef)
+        return HJ_OK;
+    int n = 0;
+    const TileKernelInfo *k = family_tiles(fam, &n);
+    for (int i = 0; i < n; ++i) {
+        if (k[i].dim != 2 || k[i].tx != h->p.tile_x || k[i].ty != h->p.tile_y) continue;
+        const PersistKernelInfo *pk = find_persist(fam, 2, k[i].tx, k[i].ty, k[i].threads);
+        int cap = 0;
+        if (pk) CKS(persist_capacity(h, pk, sig, &cap));
+        dim3 g, b;
+        geometry(h, &k[i], false, &g, &b);
+        if ((long long)g.x * g.y <= cap) {
+            *threads = k[i].threads;
+            return HJ_OK;
+        }
+    }
+    return HJ_OK;
+}
+
 // Graph of M launches of fn; launch i takes args[i % period].
 template <typename Args>
 int get_graph(hj_handle *h, void (*fn)(Args), dim3 grid, dim3 block, int smem, const Args *args, int period,
@@ -384,6 +410,9 @@ struct Plan {
 // subdomains) are about 40 us of loads and adds against launches of 130 us
 // (binary32) and more.  Beyond that the grid reduction at the launch's end stays.
 constexpr long long kDeferMaxBlocks = 65536;
+// In place, the deferred fold leaves the array two cycles past the checked one, the
+// grid reduction one: 1D runs and larger 2D grids than this keep the latter.
+constexpr long long kDeferInPlace2D = 4096;
 
 // 3D: whether the prefetching (persistent-warp, cp.async) kernel runs.  Only
 // on request (pipeline = 1): measured at 512^3 binary32 it is slower than the
@@ -474,6 +503,7 @@ bool defer_hier(const hj_handle *h, const TileKernelInfo *ki, bool classic) {
     if (classic || !ki || h->d.dim == 3 || h->d.coef) return false;
     dim3 g, b;
     geometry(h, ki, false, &g, &b);
+    if (h->p.in_place) return h->d.dim == 2 && (long long)g.x * g.y <= kDeferInPlace2D;
     return (long long)g.x * g.y <= kDeferMaxBlocks;
 }
 
@@ -882,7 +912,7 @@ int iterate(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int
                           hist_out, hist_cap, hist_len);
     }
     const PersistKernelInfo *pk =
-        classic ? nullptr : find_persist(fam, h->d.dim, ki->tx, ki->ty, ki->threads / ki->tiles_per_cta);
+        classic || ki->cluster > 1 ? nullptr : find_persist(fam, h->d.dim, ki->tx, ki->ty, ki->threads / ki->tiles_per_cta);
     PersistKernel pclassic = nullptr;
     if (classic) {
         const PersistClassicInfo *pc = fam == FAM_F64 ? persist_classic_f64()
@@ -916,7 +946,7 @@ int iterate(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int
             // 512 x 512 10.1 against 6.4 us a cycle, 64 x 64 8.8 against 6.5; 1D
             // binary64, 512 points 12.3 against 10.2)
             // (in-place runs stay: their array is one cycle past the checked one
-            // there, two with the deferred fold)
+            // there, up to two in graphs)
             use = (pclassic || h->p.in_place) && blocks <= cap;
         }
     }
@@ -1488,10 +1518,18 @@ int hj_create(hj_handle **out, const hj_desc *desc, const hj_params *params) {
             h->p.tile_threads = best;
         }
     }
+    int in_th = 0;
+    if (!p.tile_threads) {
+        st = in_place_threads(h, ir ? h->fam_inner : h->fam_outer, d.sigma != nullptr, &in_th);
+        if (st != HJ_OK) {
+            hj_destroy(h);
+            return st;
+        }
+    }
     if (d.dim == 3) {
         // kernels picked above (k3) or the classic seven-point sweep
     } else if (ir) {
-        const int th = p.tile_threads ? p.tile_threads : default_threads(h->fam_inner, d, p, h->nsm);
+        const int th = p.tile_threads ? p.tile_threads : in_th ? in_th : default_threads(h->fam_inner, d, p, h->nsm);
         h->k_inner = find_tile(h->fam_inner, d.dim, p.tile_x, p.tile_y, th);
         if (!h->k_inner)
             HJ_FAIL(HJ_ERR_UNSUPPORTED, "tile %dx%d (%d threads) not built for this precision", p.tile_x, p.tile_y,
@@ -1504,7 +1542,7 @@ int hj_create(hj_handle **out, const hj_desc *desc, const hj_params *params) {
     } else {
         // (variable coefficients run their own thread-per-point kernel: any
         // subdomain of at most 1024 points)
-        const int th = p.tile_threads ? p.tile_threads : default_threads(h->fam_outer, d, p, h->nsm);
+        const int th = p.tile_threads ? p.tile_threads : in_th ? in_th : default_threads(h->fam_outer, d, p, h->nsm);
         h->k_outer = d.coef ? nullptr : cluster_choice(h->fam_outer, d, p, h->nsm);
         if (!h->k_outer && !d.coef) h->k_outer = find_tile(h->fam_outer, d.dim, p.tile_x, p.tile_y, th);
         if (!h->k_outer && !d.coef)
