@@ -226,8 +226,10 @@ typedef struct {
                              res0 and res_final are exact residuals of the
                              initial and the returned array (which may be one
                              cycle past the checked one; two where a launch's
-                             residual is folded by the next one).  0 (default):
-                             u_c and u_{c+1} in separate arrays, deterministic */
+                             residual is folded by the next one).  k = 1 on 2D
+                             subdomains of several warps runs in two arrays.
+                             0 (default): u_c and u_{c+1} in separate arrays,
+                             deterministic                                     */
     int tile_z;           /* 3D: subdomain depth; 0 = the default 3D shape of
                              the precision (binary32 16 x 8 x 8, binary64
                              16 x 4 x 8), which replaces tile_x and tile_y.

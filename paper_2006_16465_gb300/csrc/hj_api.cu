@@ -1016,6 +1016,16 @@ cudaError_t copy_back(const hj_handle *h, void *u, const void *src, cudaStream_t
                              cudaMemcpyDeviceToDevice, s);
 }
 
+// Whether a run in place uses the one array.  With one subiteration no barrier lies
+// between one warp's staging and another's write-back, so a warp could read rows of its
+// own subdomain that are already overwritten, which is not for a neighbour's halo only:
+// subdomains of several warps run in two arrays then.
+bool one_array(const hj_handle *h, const TileKernelInfo *ki) {
+    if (!h->p.in_place) return false;
+    if (h->p.k > 1 || h->d.dim != 2 || h->p.method != HJ_METHOD_HIER) return true;
+    return h->d.coef ? !vc_rows(h) || h->p.tile_y == 4 : ki->threads * ki->cluster == 32;
+}
+
 // Plain (binary64 or binary32) solve of A u = f, u in/out (device).
 int solve_plain(hj_handle *h, const void *f, void *u, bool transpose, cudaStream_t s, hj_stats *st) {
     const bool classic = h->p.method == HJ_METHOD_CLASSIC;
@@ -1024,7 +1034,7 @@ int solve_plain(hj_handle *h, const void *f, void *u, bool transpose, cudaStream
     CycArgs base = base_args(h, transpose);
     base.f = f;
     base.dinv = h->dinv_outer;
-    const bool inplace = h->p.in_place != 0;
+    const bool inplace = one_array(h, ki);
     if (!inplace) CKR(copy_ring(h, u, h->ubuf, s));
     // in place, even the first cycle's staged data may mix u_0 and u_1: take
     // ||r_0|| exactly for the final status
@@ -1108,7 +1118,7 @@ int solve_ir(hj_handle *h, const double *f, double *u, bool transpose, cudaStrea
         if (o >= h->p.max_outer) { status = HJ_ERR_NOT_CONVERGED; break; }
         CKR(cudaMemsetAsync(h->dA, 0, (size_t)h->rows * h->ld_in * dsz, s));
         RunOut ro;
-        const bool inplace = h->p.in_place != 0;
+        const bool inplace = one_array(h, h->k_inner);
         CKS(iterate(h, h->k_inner, h->p_inner, h->fam_inner, false, sig, base, h->dA, inplace ? h->dA : h->dB,
                     ThirdBuffer{&h->dC, (size_t)h->rows * h->ld_in * dsz, (int)dsz, inplace ? h->dA : nullptr},
                     h->p.inner_tol, h->p.inner_max_cycles, 0, s, &ro, nullptr, 0, nullptr, &persist));
