@@ -190,8 +190,11 @@ typedef struct {
                              subdomain                                        */
     int tile_threads;     /* threads per subdomain (one warp per band of rows);
                              0 = the default for the tile shape and the number
-                             of subdomains; the built
-                             combinations are listed by hj_tile_variants()      */
+                             of subdomains; the built combinations are listed
+                             by hj_tile_variants().  Binary64 32 x 32
+                             subdomains also take 512 (a cluster of CTAs each,
+                             their default) while there are at most half as
+                             many as SMs                                       */
     int pipeline_stages;  /* TMA-pipelined kernel: shared-memory stages per CTA
                              (binary32 / bfloat16: 1 or 2, binary64: 2; 0 = the
                              default, the first built).  With one stage the

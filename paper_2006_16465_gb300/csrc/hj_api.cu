@@ -196,18 +196,19 @@ int default_threads(int fam, const hj_desc &d, const hj_params &p, int nsm) {
 }
 
 // Binary64 32 x 32 subdomains on a cluster of CTAs, where the caller leaves the
-// threads to the library and the grid has so few subdomains that every CTA finds
-// an SM of its own (measured beside hier2d_cluster_kernel); else null.
+// threads to the library (or asks for a cluster's 512) and the grid has so few
+// subdomains that every CTA finds an SM of its own (measured beside
+// hier2d_cluster_kernel); else null.
 const TileKernelInfo *cluster_choice(int fam, const hj_desc &d, const hj_params &p, int nsm) {
     if (fam != FAM_F64 || d.dim != 2 || p.method != HJ_METHOD_HIER || d.coef || p.persistent == 1 || p.pipeline == 1 ||
-        p.in_place || p.tile_threads || p.tile_x != 32 || p.tile_y != 32)
+        p.in_place || p.tile_x != 32 || p.tile_y != 32)
         return nullptr;
     const long long n = (long long)subdomain_count(d.nx, p.tile_x, p.overlap_x) *
                         subdomain_count(d.ny, p.tile_y, p.overlap_y);
     int cnt = 0;
     const TileKernelInfo *k = cluster_kernels_f64(&cnt);
     for (int i = 0; i < cnt; ++i)
-        if (n * k[i].cluster <= nsm) return &k[i];
+        if (n * k[i].cluster <= nsm && (!p.tile_threads || p.tile_threads == k[i].threads * k[i].cluster)) return &k[i];
     return nullptr;
 }
 

@@ -1,0 +1,50 @@
+"""Routes that the library picks by itself: a configuration that a call reports can
+be set again, and a pick kept in a file is not read under another meaning."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+import workloads as W
+from helpers import gpu_solver, to_dev
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("nx,ny,overlap", [(96, 80, 0), (256, 256, 0), (100, 100, 4)])
+def test_reported_cluster_threads_can_be_set(nx, ny, overlap):
+    """Binary64 on clusters of four and two CTAs: 512 threads a subdomain are
+    reported, and asking for them gives the same run."""
+    import torch
+    p = W.random_bc_problem(2, nx, ny, seed=5, sigma_kind="const")
+    kw = dict(precision="f64", tile_x=32, tile_y=32, k=5, overlap_x=overlap, overlap_y=overlap, fixed_cycles=6)
+    us = []
+    for threads in (0, 512):
+        s = gpu_solver(p, tile_threads=threads, **kw)
+        u = to_dev(p.u0, 2, torch.float64)
+        assert s.solve(to_dev(p.f, 2, torch.float64), u)["tile_threads"] == 512
+        s.close()
+        us.append(u)
+    assert torch.equal(us[0], us[1])
+
+
+@pytest.mark.parametrize("kw", [dict(nx=600, ny=600), dict(in_place=1), dict(pipeline=1), dict(persistent=1),
+                                dict(tile_y=16), dict(precision="f32")])
+def test_cluster_threads_are_refused_elsewhere(kw):
+    import paper_2006_16465_gb300 as hj
+    kw = dict(kw)
+    p = W.poisson2d_uniform(kw.pop("nx", 96), kw.pop("ny", 80), seed=1)
+    params = dict(precision="f64", tile_x=32, tile_y=32, tile_threads=512)
+    params.update(kw)
+    with pytest.raises(hj.HJError) as e:
+        gpu_solver(p, **params)
+    assert e.value.code == hj.HJ_ERR_UNSUPPORTED
