@@ -58,9 +58,11 @@ std::mutex g_mu;
 std::map<std::string, std::vector<int>> g_cache;
 bool g_loaded = false;
 
+// (the version changes with the meaning of what is kept: v2 lines have
+// ctas_per_sm = 0 for "as many as fit", which is the library's own cap now)
 std::string make_key(const hj_desc &d, int precision, double tol) {
     char buf[512];
-    snprintf(buf, sizeof(buf), "v2_d%d_n%dx%d_p%d_c%.9g,%.9g,%.9g,%.9g,%.9g_s%.9g_sig%d_tol%.3g", d.dim, d.nx, d.ny,
+    snprintf(buf, sizeof(buf), "v3_d%d_n%dx%d_p%d_c%.9g,%.9g,%.9g,%.9g,%.9g_s%.9g_sig%d_tol%.3g", d.dim, d.nx, d.ny,
              precision, d.cW, d.cE, d.cS, d.cN, d.cD, d.sigma_const, d.sigma ? 1 : 0, tol);
     return buf;
 }

@@ -48,3 +48,36 @@ def test_cluster_threads_are_refused_elsewhere(kw):
     with pytest.raises(hj.HJError) as e:
         gpu_solver(p, **params)
     assert e.value.code == hj.HJ_ERR_UNSUPPORTED
+
+
+_TUNE = r"""
+import os, sys
+sys.path.insert(0, os.getcwd())
+import torch
+import paper_2006_16465_gb300 as hj
+import workloads as W
+p = W.poisson2d_uniform(1400, 1300, seed=1)
+s = hj.Solver(p.st, tile_x=32, tile_y=32, k=4, precision="f32", tol=0.0, max_cycles=4, autotune=3)
+f = hj.grid_from(p.f, 2, torch.float32)
+print("PICK", s.solve(f, hj.grid_from(p.u0, 2, torch.float32), check=False)["ctas_per_sm"])
+s.close()
+"""
+
+
+def test_cached_pick_of_an_older_version_is_measured_again(tmp_path):
+    """Lines of the earlier key version kept ctas_per_sm = 0 with another meaning."""
+    cache = tmp_path / "cache.txt"
+
+    def run():
+        r = subprocess.run([sys.executable, "-c", _TUNE], cwd=ROOT, capture_output=True, text=True, timeout=300,
+                           env=dict(os.environ, HJ_AUTOTUNE_CACHE=str(cache)))
+        assert r.returncode == 0, r.stderr[-2000:]
+        return int([ln for ln in r.stdout.splitlines() if ln.startswith("PICK")][0].split()[1])
+
+    assert run() > 0
+    line = cache.read_text().splitlines()[0].split()
+    key, picks = line[0], line[1:]
+    assert run() == int(picks[2]) and len(cache.read_text().splitlines()) == 1   # the kept pick is used
+    picks[2] = "0"
+    cache.write_text(" ".join(["v2_" + key.split("_", 1)[1]] + picks) + "\n")
+    assert run() > 0
