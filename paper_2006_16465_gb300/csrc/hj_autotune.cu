@@ -352,7 +352,15 @@ extern "C" int hj_autotune(const hj_desc *desc, hj_params *params, double *predi
     const bool ir = params->precision == HJ_PREC_F32_IR || params->precision == HJ_PREC_BF16CORR_IR;
     const int prec = ir ? HJ_PREC_F32 : params->precision;   // refinement: tune the binary32 inner cycles
     const double tol = ir ? params->tol : std::max(params->tol, 1e-12);
+    // binary64 32 x 32 subdomains on clusters are a candidate where hj_create takes
+    // them (and a pick kept for such a call is not for the others)
+    int dev = 0, nsm = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const bool clusters = prec == HJ_PREC_F64 && d.dim == 2 && !params->in_place && params->persistent != 1 &&
+                          params->pipeline != 1 && 2LL * ((d.nx + 31) / 32) * ((d.ny + 31) / 32) <= nsm;
     std::string key = make_key(d, params->precision, tol);
+    if (clusters) key += "_cl";
     if (params->autotune == 2) {
         char extra[64];
         snprintf(extra, sizeof(extra), "_fixed%dx%dt%d", params->tile_x, params->tile_y, params->tile_threads);
@@ -376,7 +384,12 @@ extern "C" int hj_autotune(const hj_desc *desc, hj_params *params, double *predi
     Scratch sc;
     CKS(sc.init(d, prec));
     int xy[3 * 64];
-    const int nshape = std::min(64, hj_tile_variants(d.dim, prec, xy, 64));
+    int nshape = std::min(63, hj_tile_variants(d.dim, prec, xy, 63));
+    if (clusters) {
+        xy[3 * nshape] = xy[3 * nshape + 1] = 32;
+        xy[3 * nshape + 2] = 512;
+        ++nshape;
+    }
     const int ks[] = {4, 8, 16, 32, 64};
     const int os[] = {0, 2, 4, 8};   // overlapping points per side (Sections 3.4, 4.3)
     double best = INFINITY;

@@ -81,3 +81,17 @@ def test_cached_pick_of_an_older_version_is_measured_again(tmp_path):
     picks[2] = "0"
     cache.write_text(" ".join(["v2_" + key.split("_", 1)[1]] + picks) + "\n")
     assert run() > 0
+
+
+def test_autotune_measures_the_cluster_variant():
+    """The pick for a binary64 plane of few 32 x 32 subdomains is no slower than the
+    default (on clusters): with the shape given, it is the cluster variant; a pick for
+    an in-place run stays one that in-place runs take."""
+    import torch
+    p = W.poisson2d_uniform(128, 128, seed=1)
+    f = to_dev(p.f, 2, torch.float64)
+    for in_place, threads in ((0, (512,)), (1, (64, 128, 256))):
+        s = gpu_solver(p, precision="f64", tile_x=32, tile_y=32, tol=1e-3, autotune=2, in_place=in_place)
+        out = s.solve(f, to_dev(p.u0, 2, torch.float64))
+        s.close()
+        assert out["status"] == 0 and out["tile_threads"] in threads
