@@ -741,8 +741,8 @@ struct RunOut {
     void *buf;          // the buffer that holds iterate c
 };
 
-// Where a converging run keeps its third iterate buffer (allocated on first
-// use: only the pipelined kernel's deferred residual fold needs it).
+// Where a converging run keeps its third iterate buffer (allocated on first use:
+// the deferred residual fold needs it).
 struct ThirdBuffer {
     void **slot;
     size_t bytes;
@@ -818,12 +818,13 @@ int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, 
         b2 = third.alias;
     } else if (deferred_run(h, ki, pi, classic)) {
         if (!third.slot) return seterr(HJ_ERR_CUDA, "internal: no slot for the third iterate buffer");
-        if (!*third.slot && dmalloc(third.slot, third.bytes) != cudaSuccess) {
+        // the one-CTA-per-subdomain kernels run without it (grid reduction at a launch's end)
+        const bool need = want_ppc(h, pi, classic) || want_ppc3(h, classic);
+        if (!*third.slot && (need || !h->no_third) && dmalloc(third.slot, third.bytes) != cudaSuccess) {
             cudaGetLastError();
             *third.slot = nullptr;
-            // the one-CTA-per-subdomain kernels run without it (grid reduction at a launch's end)
-            if (want_ppc(h, pi, classic) || want_ppc3(h, classic))
-                return seterr(HJ_ERR_NO_MEMORY, "third iterate buffer (%zu bytes)", third.bytes);
+            if (need) return seterr(HJ_ERR_NO_MEMORY, "third iterate buffer (%zu bytes)", third.bytes);
+            h->no_third = true;
         }
         b2 = *third.slot;
         if (b2)

@@ -612,21 +612,28 @@ int batched_core(hj_handle *h, int nprob, const hj_desc *descs, const void *cons
         thirds += (b.nin * dsz + 255) / 256 * 256;
         if (sig_any) arena += (b.nin * 4 + 255) / 256 * 256;          // per-point 1/d (binary32)
     }
+    // without the third correction buffers the plain-staging engine runs
+    auto without_thirds = [&]() {
+        arena -= thirds;
+        thirds = 0;
+    };
+    if (arena > h->barena_bytes && h->barena_refused && arena >= h->barena_refused) without_thirds();
     if (arena > h->barena_bytes) {
         CKR(cudaDeviceSynchronize());
         if (h->barena) dfree(h->barena);
         h->barena = nullptr;
         h->barena_bytes = 0;
-        if (dmalloc(&h->barena, arena) != cudaSuccess) {
-            // without the third correction buffers the plain-staging engine runs
+        cudaError_t e = dmalloc(&h->barena, arena);
+        if (e != cudaSuccess && thirds) {
             cudaGetLastError();
-            arena -= thirds;
-            thirds = 0;
-            if (dmalloc(&h->barena, arena) != cudaSuccess) {
-                cudaGetLastError();
-                h->barena = nullptr;
-                return seterr(HJ_ERR_NO_MEMORY, "batched workspace of %zu bytes", arena);
-            }
+            h->barena_refused = h->barena_refused ? std::min(h->barena_refused, arena) : arena;
+            without_thirds();
+            e = dmalloc(&h->barena, arena);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            h->barena = nullptr;
+            return seterr(HJ_ERR_NO_MEMORY, "batched workspace of %zu bytes", arena);
         }
         h->barena_bytes = arena;
     }

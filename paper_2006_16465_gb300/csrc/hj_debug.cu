@@ -6,9 +6,13 @@
 //     exchange and write-back indices (HJ_IN) and record the first failure
 //     here instead of trapping;
 //   * hj_debug_check reports both, hj_debug_selftest shows that each is
-//     caught, without touching memory out of bounds.
+//     caught, without touching memory out of bounds;
+//   * HJ_TEST_ALLOC_LIMIT (bytes) refuses larger allocations, as a full device
+//     would, and says so on stderr: the tests of what runs without a buffer.
 // Release builds allocate with plain cudaMalloc / cudaFree, compile the index
 // checks away, and hj_debug_check reports that no checks are compiled in.
+#include <cstdio>
+#include <cstdlib>
 #include <map>
 #include <mutex>
 
@@ -65,6 +69,13 @@ __global__ void debug_selftest_kernel(DbgWord *w) {
 
 cudaError_t dmalloc(void **p, size_t bytes) {
 #ifdef HJ_DEBUG
+    if (const char *lim = getenv("HJ_TEST_ALLOC_LIMIT")) {
+        if (*lim && bytes > (size_t)atoll(lim)) {
+            fprintf(stderr, "HJ_TEST_ALLOC_LIMIT: %zu bytes refused\n", bytes);
+            *p = nullptr;
+            return cudaErrorMemoryAllocation;
+        }
+    }
     unsigned char *base = nullptr;
     cudaError_t e = cudaMalloc((void **)&base, bytes + 2 * kGuard);
     if (e != cudaSuccess) {

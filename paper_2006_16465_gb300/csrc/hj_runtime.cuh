@@ -84,7 +84,8 @@ struct hj_handle {
     const hj::Tile3Info *k3 = nullptr;                                 // 3D seven-point kernel (hierarchical)
     long long ld_in = 0;          // row pitch of the refinement's binary32 / bfloat16 arrays
     void *ubuf = nullptr;
-    void *ubuf2 = nullptr;        // third iterate buffer (pipelined kernel, deferred residual fold)
+    void *ubuf2 = nullptr;        // third iterate buffer (deferred residual fold)
+    bool no_third = false;        // a third buffer could not be had: runs that can do without do not ask again
     float *vcf = nullptr;         // binary32 factors of the variable-coefficient kernels
     void *dinv_outer = nullptr;   // per-point 1/d in the outer compute type (sigma given)
     float *dinv32 = nullptr;      // per-point 1/d in binary32 (refinement, sigma given)
@@ -110,6 +111,7 @@ struct hj_handle {
     // batched solves: per-problem arrays and norms
     void *barena = nullptr;
     size_t barena_bytes = 0;
+    size_t barena_refused = 0;   // smallest workspace with third correction buffers that could not be had (0: none)
     double *rs = nullptr, *h_rs = nullptr;
     size_t nrs = 0;
     // batched solves: device metadata of the batch (per-problem buffers and
