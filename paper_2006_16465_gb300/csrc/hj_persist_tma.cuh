@@ -201,7 +201,8 @@ __device__ __forceinline__ void batch_queue_rebuild(const PersistArgs &P) {
         const int off = P.q_off[p];
         if (off < 0) continue;
         const int i0 = P.prob_item0[p], n = P.prob_nitems[p], tx = P.prob_tiles_x[p];
-        for (int b = threadIdx.x; b < n; b += blockDim.x) P.q_ent[off + b] = make_int4(i0 + b, p, b % tx, b / tx);
+        for (int b = threadIdx.x; b < n; b += blockDim.x)
+            if (HJ_IN(P.probs[0].dbg, off + b, P.nitems, 52)) P.q_ent[off + b] = make_int4(i0 + b, p, b % tx, b / tx);
     }
 }
 
@@ -324,6 +325,15 @@ __global__ void __launch_bounds__(32 * NW, (NW == 4 && SIG) ? 3 : 0) persist2d_b
     const int me = cta_rank(P.sm_ctas, (int)sm, s_slot);
     int4 first = make_int4(0, 0, 0, 0);
     int first_of = head.w - 1;   // the rebuild `first` was read from
+    // entry i of the queue; debug builds check what a wrong one would send copies and
+    // stores out of range with
+    auto entry = [&](int i) -> int4 {
+        if (!HJ_IN(P.probs[0].dbg, i, P.nitems, 51)) return make_int4(0, 0, 0, 0);
+        const int4 e = __ldcg(P.q_ent + i);
+        if (!HJ_IN(P.probs[0].dbg, e.x, P.nitems, 51) || !HJ_IN(P.probs[0].dbg, e.y, P.nprob, 51))
+            return make_int4(0, 0, 0, 0);
+        return e;
+    };
     // every active problem advances once per cycle: `it` is its cycle index
     for (long long it = 0; it < P.max_iters; ++it) {
         const int cnt = head.x, alive = head.z, total = cnt + (it > 0 ? head.y : 0);
@@ -338,7 +348,7 @@ __global__ void __launch_bounds__(32 * NW, (NW == 4 && SIG) ? 3 : 0) persist2d_b
         };
         int i = me;
         if (first_of != head.w) {
-            if (i < cnt) first = __ldcg(P.q_ent + i);
+            if (i < cnt) first = entry(i);
             first_of = head.w;
         }
         int4 e = first, en = first;
@@ -350,7 +360,7 @@ __global__ void __launch_bounds__(32 * NW, (NW == 4 && SIG) ? 3 : 0) persist2d_b
             }
             if (total > alive) {
                 nidx = atomicAdd(P.q_head, 1);
-                if (nidx < cnt) en = __ldcg(P.q_ent + nidx);
+                if (nidx < cnt) en = entry(nidx);
             }
         }
         while (i < cnt) {
@@ -406,7 +416,7 @@ __global__ void __launch_bounds__(32 * NW, (NW == 4 && SIG) ? 3 : 0) persist2d_b
             if (tid == 0 && HJ_IN(a.dbg, pi, 2 * (long long)P.nitems, 50)) P.partial[pi] = s;
             if (tid == 0) {
                 nidx = after;
-                if (nidx < cnt) en = __ldcg(P.q_ent + nidx);
+                if (nidx < cnt) en = entry(nidx);
             }
             i = inext;
             e = enext;
