@@ -748,14 +748,16 @@ struct ThirdBuffer {
     size_t bytes;
     int esz;       // element size
     void *alias;   // in-place runs: every iterate buffer is this array
+    bool ringed = false;   // the buffer, if there is one, has b0's ghost ring already
 };
 
 // Iterate cycles (or classic sweeps) from b0 (holds u_0) and b1 (the other
 // buffer, same ghost ring).  fixed > 0: exactly `fixed` cycles, no residual.
-// Otherwise until ||r_c|| <= tol ||r_0|| or max_cycles.
+// Otherwise until ||r_c|| <= tol ||r_0|| or max_cycles; ramp >= 0: with the first
+// checks early, after about `ramp` cycles where it is not 0.
 int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int fam, bool classic, bool sig,
                const CycArgs &base_in, void *b0, void *b1, ThirdBuffer third, double tol, long long max_cycles,
-               long long fixed, cudaStream_t s, RunOut *ro, double *hist_out, long long hist_cap,
+               long long fixed, long long ramp, cudaStream_t s, RunOut *ro, double *hist_out, long long hist_cap,
                long long *hist_len) {
     int M = h->p.check_every;
     ro->res2_0 = -1.0;
@@ -820,14 +822,17 @@ int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, 
         if (!third.slot) return seterr(HJ_ERR_CUDA, "internal: no slot for the third iterate buffer");
         // the one-CTA-per-subdomain kernels run without it (grid reduction at a launch's end)
         const bool need = want_ppc(h, pi, classic) || want_ppc3(h, classic);
-        if (!*third.slot && (need || !h->no_third) && dmalloc(third.slot, third.bytes) != cudaSuccess) {
-            cudaGetLastError();
-            *third.slot = nullptr;
-            if (need) return seterr(HJ_ERR_NO_MEMORY, "third iterate buffer (%zu bytes)", third.bytes);
-            h->no_third = true;
+        if (!*third.slot && (need || !h->no_third)) {
+            third.ringed = false;
+            if (dmalloc(third.slot, third.bytes) != cudaSuccess) {
+                cudaGetLastError();
+                *third.slot = nullptr;
+                if (need) return seterr(HJ_ERR_NO_MEMORY, "third iterate buffer (%zu bytes)", third.bytes);
+                h->no_third = true;
+            }
         }
         b2 = *third.slot;
-        if (b2)
+        if (b2 && !third.ringed)
             CKR(launch_copy_ring(h->d.dim, third.esz, b0, b2, nullptr, base.ld, base.ps, h->d.nx, h->d.ny, h->d.nz, s));
     }
     Plan pl;
@@ -835,16 +840,14 @@ int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, 
     // residual of launch c's input is known after launch c + 1 (deferred fold)
     const int lag = pl.deferred ? 1 : 0;
     if (pl.deferred) M = (M + kPpcPeriod - 1) / kPpcPeriod * kPpcPeriod;
-    cudaGraphExec_t ex;
-    CKS(plan_graph(h, pl, M, &ex));
+    const long long need = max_cycles + lag;   // launches that settle max_cycles
     const long long mask = kHistCap - 1;
-    // Replays are pipelined two deep: replay i+1 is queued before the host
-    // waits for replay i's control block, so the GPU does not idle while the
-    // host checks.  Replay r copies its control block into slot r % 2 and the
-    // entries of the residual ring it may have written into the pinned ring.
-    // No replay starts beyond the launch that settles max_cycles, and launches
-    // after convergence return at once.
-    long long issued = 0;   // replays queued
+    // A check copies the control block into slot r % 2 and, where the caller wants the
+    // history, the entries of the residual ring that the launches before it may have
+    // written into the pinned ring.  Launches after convergence return at once.
+    cudaGraphExec_t few = nullptr, many = nullptr;   // graphs of kPpcPeriod and of M launches
+    long long issued = 0, checked = 0, launched = 0, copied = 0;
+    const Ctl *last = nullptr;
     auto copy_ring = [&](long long lo, long long n) -> int {
         while (n > 0) {
             const long long p0 = lo & mask;
@@ -855,44 +858,84 @@ int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, 
         }
         return HJ_OK;
     };
-    auto issue = [&]() -> int {
-        const long long r = issued;
-        CKR(cudaGraphLaunch(ex, s));
-        const long long lo = std::max(0LL, r * M - lag);
-        CKS(copy_ring(lo, (r + 1) * M - lo));
-        CKR(cudaMemcpyAsync(h->h_ctl + (r & 1), h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
-        CKR(cudaEventRecord(h->evs[r & 1], s));
+    // queue launches (reps replays of the graph of n, or n single ones without it) and
+    // one check of them
+    auto issue = [&](cudaGraphExec_t ex, long long n, long long reps) -> int {
+        const long long lo = std::max(0LL, launched - lag);
+        for (long long r = 0; r < reps; ++r) {
+            if (ex) CKR(cudaGraphLaunch(ex, s));
+            else
+                for (long long c = 0; c < n; ++c) plan_launch(pl, launched + c, s);
+            launched += n;
+        }
+        CKR(cudaGetLastError());
+        if (hist_out) CKS(copy_ring(lo, launched - lo));
+        CKR(cudaMemcpyAsync(h->h_ctl + (issued & 1), h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
+        CKR(cudaEventRecord(h->evs[issued & 1], s));
         ++issued;
         return HJ_OK;
     };
-    CKS(issue());
-    long long copied = 0, checked = 0;
-    const Ctl *last = nullptr;
-    for (;;) {
-        if (issued * M < max_cycles + lag) CKS(issue());
+    // wait for the oldest check
+    auto settle = [&](bool *done) -> int {
         CKR(cudaEventSynchronize(h->evs[checked & 1]));
         last = h->h_ctl + (checked & 1);
         ++checked;
         if (last->err) return seterr(HJ_ERR_TIMEOUT, "a bounded device wait expired (tile pipeline)");
-        const long long ncomp = last->cycle;
         if (hist_out) {
-            for (; copied < ncomp; ++copied)
+            for (; copied < last->cycle; ++copied)
                 if (copied < hist_cap) hist_out[copied] = sqrt(h->h_hist[copied & mask]);
         }
-        if (last->done >= 0) break;
-        if (checked >= issued)
-            return seterr(HJ_ERR_CUDA, "cycle loop did not terminate (device control block not updated)");
+        *done = last->done >= 0;
+        return HJ_OK;
+    };
+    bool done = false;
+    // Checks are queued two deep: the launches behind the next check are queued before
+    // the host waits for this one's control block, so the GPU does not idle meanwhile.
+    // Small grids start with short graphs: a launch that returns at once still takes
+    // some 2 us, so a solve of a few cycles would pay more for what a graph of M
+    // launches, and the one queued behind it, has left than for its cycles (and for
+    // making that graph on a handle's first call).  A check costs some 25 us where
+    // nothing is queued behind it: the first is waited for so, then the launches
+    // between checks grow with those done.  64 x 64 binary32, k = 4, to 0.5 ||r_0|| (2
+    // cycles): 280 us with graphs of 64, 69 so, 70 with the persistent engine.
+    if (ramp >= 0) {
+        const long long P = kPpcPeriod;
+        if (need > 4) CKS(plan_graph(h, pl, P, &few));
+        if (!few) CKS(issue(few, need, 1));   // (single launches where there are few)
+        else CKS(issue(few, P, (std::min(ramp + lag + 1, need) + P - 1) / P));
+        CKS(settle(&done));
+        // replays before the next check, and whether the graph of M serves it better
+        auto reps = [&]() { return std::max(1LL, std::min(2 * launched, 3 * (need - launched)) / (3 * P)); };
+        auto more = [&]() { return launched < need && reps() * P < M; };
+        if (!done && more()) CKS(issue(few, P, reps()));
+        while (!done && checked < issued) {
+            if (more()) CKS(issue(few, P, reps()));
+            CKS(settle(&done));
+        }
     }
-    // the replay queued behind the converged one returns at once; wait for it
-    // so that no copy into the pinned slots is still pending when we return
+    // the next replay; no replay starts beyond the launch that settles max_cycles
+    auto next = [&]() -> int {
+        if (few && need - launched < M) return issue(few, kPpcPeriod, (need - launched + kPpcPeriod - 1) / kPpcPeriod);
+        if (!many) CKS(plan_graph(h, pl, M, &many));
+        return issue(many, M, 1);
+    };
+    if (!done && launched < need) {
+        CKS(next());
+        while (!done && checked < issued) {
+            if (launched < need) CKS(next());
+            CKS(settle(&done));
+        }
+    }
+    // what is queued behind the converged run returns at once; wait for it so that no
+    // copy into the pinned slots is still pending when we return
     if (issued > checked) CKR(cudaEventSynchronize(h->evs[(issued - 1) & 1]));
-    const long long launched = issued * M;   // kernels launched, including returns-at-once overshoot
+    if (!done) return seterr(HJ_ERR_CUDA, "cycle loop did not terminate (device control block not updated)");
     if (hist_len) *hist_len = std::min(copied, hist_cap);
     ro->c = last->done;
     ro->status = last->status;
     ro->launched = launched;
     ro->res2_0 = last->res2_0;
-    if (ro->status == HJ_OK || ro->status == HJ_ERR_DIVERGED) ro->res2_c = h->h_hist[ro->c & mask];
+    if (ro->status == HJ_OK || ro->status == HJ_ERR_DIVERGED) ro->res2_c = last->res2_last;
     if (pl.deferred) {
         void *bufs[3] = {b0, b1, b2};
         ro->buf = bufs[ro->c % 3];
@@ -902,15 +945,16 @@ int run_cycles(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, 
     return HJ_OK;
 }
 
-// Iterate with the persistent engine when every block of the grid can be
-// resident at once (or when forced), else with graph-captured launches.
+// Iterate with the persistent engine where it is forced, and for classic and
+// in-place runs when every block of the grid can be resident at once; else with
+// launches (run_cycles).  expect: about how many cycles it will take (0: unknown).
 int iterate(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int fam, bool classic, bool sig,
             const CycArgs &base, void *b0, void *b1, ThirdBuffer third, double tol, long long max_cycles,
             long long fixed, cudaStream_t s, RunOut *ro, double *hist_out, long long hist_cap, long long *hist_len,
-            int *used_persistent) {
+            int *used_persistent, long long expect = 0) {
     if (h->d.coef || h->d.dim == 3) {   // variable coefficients and 3D: graph-captured launches only
         if (used_persistent) *used_persistent = 0;
-        return run_cycles(h, ki, pi, fam, classic, sig, base, b0, b1, third, tol, max_cycles, fixed, s, ro,
+        return run_cycles(h, ki, pi, fam, classic, sig, base, b0, b1, third, tol, max_cycles, fixed, -1, s, ro,
                           hist_out, hist_cap, hist_len);
     }
     const PersistKernelInfo *pk =
@@ -927,7 +971,17 @@ int iterate(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int
     const long long cblocks = h->d.dim == 2 ? (long long)((h->d.nx + 31) / 32) * ((h->d.ny + 7) / 8)
                                             : (long long)((h->d.nx + 255) / 256) * h->d.ny;
     bool use = false;
-    if ((pk || pclassic) && fixed <= 0 && max_cycles > 0 && h->p.persistent != 0 && !overlapped(h) && !h->d.coef) {
+    long long ramp = -1;
+    if (!classic && !h->p.in_place && h->p.persistent == -1 && fixed <= 0 && max_cycles > 0 && !overlapped(h)) {
+        // (the grids that one wave of persistent CTAs could hold; at tol = 0 the cap ends
+        // the run)
+        if (tol == 0.0) expect = max_cycles;
+        const PersistKernelInfo *p0 = pk ? pk : find_persist(fam, h->d.dim, ki->tx, ki->ty, 0);
+        int cap = 0;
+        if (p0) CKS(persist_capacity(h, p0, sig, &cap));
+        if ((long long)g.x * g.y / ki->cluster <= cap && expect < std::min(4LL * h->p.check_every, 1024LL))
+            ramp = expect;
+    } else if ((pk || pclassic) && fixed <= 0 && max_cycles > 0 && h->p.persistent != 0 && !overlapped(h) && !h->d.coef) {
         int cap = 0;
         if (pclassic) {
             int occ = 0;
@@ -941,7 +995,7 @@ int iterate(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int
             if (blocks > 64LL * cap) return seterr(HJ_ERR_UNSUPPORTED, "grid too large for the persistent engine");
             use = true;
         } else {
-            // hierarchical cycles run as graphs of launches: a kernel boundary
+            // hierarchical cycles run as launches (above): a kernel boundary
             // inside a graph costs 1.0 us on this part, a grid barrier 1.5 to 2.5
             // us and the decision behind it another 1.5, where the graph's fold
             // runs beside the sweeps (32 x 32, k = 32, binary32 cycles:
@@ -954,7 +1008,7 @@ int iterate(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, int
     }
     if (used_persistent) *used_persistent = use ? 1 : 0;
     if (!use)
-        return run_cycles(h, ki, pi, fam, classic, sig, base, b0, b1, third, tol, max_cycles, fixed, s, ro,
+        return run_cycles(h, ki, pi, fam, classic, sig, base, b0, b1, third, tol, max_cycles, fixed, ramp, s, ro,
                           hist_out, hist_cap, hist_len);
     std::vector<PersistProblem> v(1);
     PersistProblem &q = v[0];
@@ -1008,8 +1062,9 @@ int residual_of(hj_handle *h, const void *f, const void *u, bool transpose, doub
 // The second iterate buffer's ghost ring, and an iterate that ended in another
 // buffer back into the caller's array (padding columns stay the caller's).
 // Whole-array copies took 80 us (8192 x 8192 binary32) to 160 us (512^3) each.
-cudaError_t copy_ring(const hj_handle *h, const void *u, void *dst, cudaStream_t s) {
-    return launch_copy_ring(h->d.dim, (int)h->esz, u, dst, nullptr, h->d.ld, (long long)(h->d.ny + 2) * h->d.ld, h->d.nx,
+// also (nullable): the third buffer, in the same launch.
+cudaError_t copy_ring(const hj_handle *h, const void *u, void *dst, void *also, cudaStream_t s) {
+    return launch_copy_ring(h->d.dim, (int)h->esz, u, dst, also, h->d.ld, (long long)(h->d.ny + 2) * h->d.ld, h->d.nx,
                             h->d.ny, h->d.nz, s);
 }
 cudaError_t copy_back(const hj_handle *h, void *u, const void *src, cudaStream_t s) {
@@ -1037,7 +1092,7 @@ int solve_plain(hj_handle *h, const void *f, void *u, bool transpose, cudaStream
     base.f = f;
     base.dinv = h->dinv_outer;
     const bool inplace = one_array(h, ki);
-    if (!inplace) CKR(copy_ring(h, u, h->ubuf, s));
+    if (!inplace) CKR(copy_ring(h, u, h->ubuf, h->p.fixed_cycles > 0 ? nullptr : h->ubuf2, s));
     // in place, even the first cycle's staged data may mix u_0 and u_1: take
     // ||r_0|| exactly for the final status
     double r0_exact = -1.0;
@@ -1050,7 +1105,7 @@ int solve_plain(hj_handle *h, const void *f, void *u, bool transpose, cudaStream
     long long hl = 0;
     int persist = 0;
     CKS(iterate(h, ki, classic ? nullptr : h->p_outer, h->fam_outer, classic, sig, base, u, inplace ? u : h->ubuf,
-                ThirdBuffer{&h->ubuf2, h->grid_bytes, (int)h->esz, inplace ? u : nullptr}, h->p.tol, h->p.max_cycles,
+                ThirdBuffer{&h->ubuf2, h->grid_bytes, (int)h->esz, inplace ? u : nullptr, !inplace}, h->p.tol, h->p.max_cycles,
                 h->p.fixed_cycles, s, &ro, st ? st->history : nullptr, st ? st->history_cap : 0, &hl, &persist));
     if (ro.buf != u) CKR(copy_back(h, u, ro.buf, s));
     double res0 = -1.0, resc = -1.0;
@@ -1093,7 +1148,7 @@ int solve_ir(hj_handle *h, const double *f, double *u, bool transpose, cudaStrea
     const CycArgs geo = base_args(h, transpose);
     const bool bf16 = h->fam_inner == FAM_BF16;
     const size_t dsz = bf16 ? 2 : 4;
-    CKR(copy_ring(h, u, h->ubuf, s));
+    CKR(copy_ring(h, u, h->ubuf, nullptr, s));
     // outer residual of u_0 -> r32
     {
         const RedArgs red = red_args(h, RED_STORE, 0.0, 0);
@@ -1106,6 +1161,7 @@ int solve_ir(hj_handle *h, const double *f, double *u, bool transpose, cudaStrea
     double *cur = u, *other = (double *)h->ubuf;
     double r0 = sqrt(h->h_rstore[0]), rn = r0;
     long long inner_total = 0, inner_launched = 0;
+    long long expect = 24;   // cycles of the next inner solve, about (to 1e-4 rarely fewer; then as the last one took)
     int o = 0, status = HJ_OK, persist = 0;
     long long hl = 0;
     CycArgs base = geo;
@@ -1113,6 +1169,7 @@ int solve_ir(hj_handle *h, const double *f, double *u, bool transpose, cudaStrea
     base.f = h->r32;
     base.dinv = h->dinv32;
     base.red.stall_window = h->p.inner_stall;
+    bool ringed = h->dC != nullptr;   // (the ghost ring of the corrections is zero and never written)
     for (;; ++o) {
         if (st && st->history && o < st->history_cap) { st->history[o] = rn; hl = o + 1; }
         if (!std::isfinite(rn)) { status = HJ_ERR_DIVERGED; break; }
@@ -1122,8 +1179,10 @@ int solve_ir(hj_handle *h, const double *f, double *u, bool transpose, cudaStrea
         RunOut ro;
         const bool inplace = one_array(h, h->k_inner);
         CKS(iterate(h, h->k_inner, h->p_inner, h->fam_inner, false, sig, base, h->dA, inplace ? h->dA : h->dB,
-                    ThirdBuffer{&h->dC, (size_t)h->rows * h->ld_in * dsz, (int)dsz, inplace ? h->dA : nullptr},
-                    h->p.inner_tol, h->p.inner_max_cycles, 0, s, &ro, nullptr, 0, nullptr, &persist));
+                    ThirdBuffer{&h->dC, (size_t)h->rows * h->ld_in * dsz, (int)dsz, inplace ? h->dA : nullptr, ringed},
+                    h->p.inner_tol, h->p.inner_max_cycles, 0, s, &ro, nullptr, 0, nullptr, &persist, expect));
+        expect = ro.c;
+        ringed = h->dC != nullptr;
         inner_total += ro.c;
         inner_launched += ro.launched;
         const void *dsel = ro.buf;

@@ -1,0 +1,49 @@
+"""Both sides of the rules by which a call takes one kernel or another, at the sizes
+around their lines: the same iterates and cycle counts, or the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+from helpers import gpu_solver, rel_max, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+def _dt(prec):
+    import torch
+    return torch.float32 if prec == "f32" else torch.float64
+
+
+def _solve(p, dim, history=0, **kw):
+    s = gpu_solver(p, **kw)
+    u = to_dev(p.u0, dim, _dt(kw["precision"]))
+    out = s.solve(to_dev(p.f, dim, _dt(kw["precision"])), u, history=history, check=False)
+    s.close()
+    return out, to_host(u, p.st.nx)
+
+
+@pytest.mark.parametrize("prec,tile,n", [("f64", (32, 32), (96, 80)), ("f64", (32, 8), (70, 45)), ("f32", (32, 32), (200, 130)),
+                                          ("f32", (32, 16), (64, 64)), ("f64", (128, 1), (300, 3))])
+def test_short_solves_equal_the_persistent_engine(prec, tile, n):
+    """Small grids run their first 48 launches singly, checked in short runs, then
+    graphs: every cycle cap around those lengths, and tolerances met within them."""
+    dim = 1 if tile[1] == 1 else 2
+    p = W.random_bc_problem(dim, *n, seed=17, sigma_kind="const")
+    base = dict(precision=prec, tile_x=tile[0], tile_y=tile[1], k=3)
+    runs = [dict(tol=0.0, max_cycles=m) for m in (1, 2, 3, 4, 5, 6, 7, 11, 12, 13, 46, 47, 48, 49, 66, 113, 114, 115, 200)]
+    runs += [dict(tol=t, max_cycles=100000) for t in (1.0, 0.9, 0.5, 0.2, 0.1, 0.05, 0.02, 0.01)]
+    for kw in runs:
+        a, ua = _solve(p, dim, history=300, persistent=-1, **base, **kw)
+        b, ub = _solve(p, dim, history=300, persistent=1, pipeline=0, **base, **kw)
+        assert (a["persistent"], b["persistent"]) == (0, 1)
+        assert (a["status"], a["cycles"]) == (b["status"], b["cycles"]), kw
+        assert np.array_equal(ua, ub), kw
+        assert a["history_len"] == b["history_len"] and np.allclose(a["history"], b["history"], rtol=1e-6, atol=0), kw
+        assert a["rel_final"] == pytest.approx(b["rel_final"], rel=1e-6), kw
