@@ -405,12 +405,27 @@ struct Plan {
     PpcArgs p[kPpcPeriod];
 };
 
-// Largest grid of the one-CTA-per-subdomain kernels that folds its residual
-// in the next launch.  A CTA of its own folds while the others sweep, in less
-// time than they take at any size: 65,536 partials (8192 x 8192 in 32 x 32
-// subdomains) are about 40 us of loads and adds against launches of 130 us
-// (binary32) and more.  Beyond that the grid reduction at the launch's end stays.
-constexpr long long kDeferMaxBlocks = 65536;
+// Largest grid (in CTAs) of the one-CTA-per-subdomain kernels that folds its residual
+// in the next launch.  A CTA of its own folds while the others sweep, at some 3 ns a
+// partial (a chain of loads from L2, 128 partials a step); beyond the limit that is
+// longer than the launch, which the grid reduction at a launch's end then serves
+// better.  Measured, us a cycle with the reduction and with the fold: binary32, k = 1,
+// 32 x 8 subdomains: 2048 x 2048 (16,384 CTAs) 23.6, 33.1, 1024 x 1024 overlapping
+// (5,800) 15.3, 17.2; 32 x 16: 2048 x 2048 (8,192) 20.5, 18.9, 3000 x 3000 (17,700)
+// 37.9, 48.1; 32 x 32: 4096 x 4096 (16,384) 55.0, 52.2 and overlapping 75.5, 60.6,
+// 8192 x 8192 (65,536) 185, 196; lines, k = 16, 64-point subdomains: 8,000 CTAs 24.1,
+// 22.4, 128-point ones: 8,000 24.1, 21.2, 32,000 76.6, 82.7, 256-point ones: 30,000
+// 80.1, 71.8, 128-point ones with a sigma field 16,000 52.5, 45.8, overlapping 63.8,
+// 61.8.  Binary64 (FP64-bound launches): 32 x 8, k = 1, 4096 x 4096 (65,536) 417, 386.
+long long defer_max_blocks(const hj_handle *h, long long blocks) {
+    if ((h->ir ? h->fam_inner : h->fam_outer) == FAM_F64) return 65536;
+    const long long pts = ((long long)h->d.nx * h->d.ny + blocks - 1) / blocks;   // points of a CTA (about)
+    if (h->d.dim == 1) {
+        const bool longer = h->p.tile_x >= (h->d.sigma || overlapped(h) ? 128 : 256);
+        return pts >= 200 ? (longer ? 32768 : 8192) : 4096;
+    }
+    return pts >= 1800 ? 65536 : pts >= 700 ? 32768 : pts >= 400 ? 8192 : 4096;
+}
 // In place, the deferred fold leaves the array two cycles past the checked one, the
 // grid reduction one: 1D runs and larger 2D grids than this keep the latter.
 constexpr long long kDeferInPlace2D = 4096;
@@ -499,13 +514,13 @@ bool want_ppc(const hj_handle *h, const PpcKernelInfo *pi, bool classic) {
 // Whether a converging run of the one-CTA-per-subdomain kernels folds its
 // residual in the next launch (as the pipelined kernel always does): 1D and 2D
 // hierarchical cycles with constant coefficients on grids of at most
-// kDeferMaxBlocks CTAs.
+// defer_max_blocks CTAs.
 bool defer_hier(const hj_handle *h, const TileKernelInfo *ki, bool classic) {
     if (classic || !ki || h->d.dim == 3 || h->d.coef) return false;
     dim3 g, b;
     geometry(h, ki, false, &g, &b);
     if (h->p.in_place) return h->d.dim == 2 && (long long)g.x * g.y <= kDeferInPlace2D;
-    return (long long)g.x * g.y <= kDeferMaxBlocks;
+    return (long long)g.x * g.y <= defer_max_blocks(h, (long long)g.x * g.y);
 }
 
 // Whether a converging run of this plan needs the third iterate buffer.

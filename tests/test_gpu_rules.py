@@ -47,3 +47,15 @@ def test_short_solves_equal_the_persistent_engine(prec, tile, n):
         assert np.array_equal(ua, ub), kw
         assert a["history_len"] == b["history_len"] and np.allclose(a["history"], b["history"], rtol=1e-6, atol=0), kw
         assert a["rel_final"] == pytest.approx(b["rel_final"], rel=1e-6), kw
+
+
+@pytest.mark.parametrize("prec,tile,n", [("f32", (32, 32), (2200, 2080)), ("f32", (32, 16), (1500, 2600)), ("f32", (32, 8), (1100, 1000)),
+                                          ("f64", (32, 8), (1100, 1000)), ("f32", (32, 16), (3000, 1500))])
+def test_folds_of_many_ctas_equal_the_pipelined_kernel(prec, tile, n):
+    """One partial per CTA, 4,000 to 9,000 of them, folded in the next launch or (the
+    last case and 32 x 8) reduced at the launch's end."""
+    p = W.random_bc_problem(2, *n, seed=8, sigma_kind="const")
+    res = [_solve(p, 2, precision=prec, tile_x=tile[0], tile_y=tile[1], k=2, tol=2e-2, check_every=6, pipeline=pl, persistent=0)
+           for pl in (0, 1)]
+    (a, ua), (b, ub) = res
+    assert a["status"] == 0 and a["cycles"] == b["cycles"] and np.array_equal(ua, ub)
