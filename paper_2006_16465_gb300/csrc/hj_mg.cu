@@ -307,14 +307,11 @@ __global__ void __launch_bounds__(1024 / RPT, (RPT == 1 && STAGE == MG_PLAIN) ? 
             }
             return nv;
         };
-        // Long runs (the coarsest level's) end at their fixed point: once a
-        // subiteration leaves every value as it was, bit for bit, so do all that
-        // follow.  A level of one point is there after two of its 256 (79 us of a
-        // V-cycle in binary64).
-        const bool watch = a.k >= 16;
-        for (int s = 0; s < a.k; ++s) {
-            const T *src = (s & 1) ? buf1 : buf0;
-            T *dst = (s & 1) ? buf0 : buf1;
+        // one subiteration; WATCH: true once it leaves every value of the CTA as it was
+        const T *src = buf0;
+        T *dst = buf1;
+        auto step = [&](int s, auto watch_tag) -> bool {
+            constexpr bool WATCH = decltype(watch_tag)::value;
             const bool more = s + 1 < a.k;   // the last subiteration's values go to global memory from registers
             T nv[RPT], prod[RPT];
             unsigned bad = 0;
@@ -335,14 +332,31 @@ __global__ void __launch_bounds__(1024 / RPT, (RPT == 1 && STAGE == MG_PLAIN) ? 
 #pragma unroll
             for (int m = 0; m < RPT; ++m) {
                 if (!in[m]) continue;
-                changed = changed || bits_differ(nv[m], v0[m]);
+                if constexpr (WATCH) changed = changed || bits_differ(nv[m], v0[m]);
                 v0[m] = nv[m];
                 if (more) dst[(ty + m * BY + 1) * lw + tx + 1] = prod[m];
             }
-            if (more) {
-                if (!watch) __syncthreads();
-                else if (!__syncthreads_or(changed)) break;
-            }
+            if (!more) return false;
+            const T *t = src;
+            src = dst;
+            dst = const_cast<T *>(t);
+            if constexpr (WATCH) return !__syncthreads_or(changed);
+            __syncthreads();
+            return false;
+        };
+        // Long runs (the coarsest level's) end at their fixed point: once a
+        // subiteration leaves every value as it was, bit for bit, so do all that
+        // follow.  A level of one point is there after two of its 256 (79 us of a
+        // V-cycle in binary64).  Binary32 looks after 2, 8, 32 subiterations and every
+        // 64 from there, in a body of its own: the comparison and the vote cost 75 ns a
+        // subiteration (6 V-cycles of 63 x 63 with a coarsest level of 15 x 15, which
+        // is never there: 263 us without, 376 with one in every subiteration, 276 so).
+        int s = 0;
+        for (int w = a.k < 16 ? a.k : EXACT ? 0 : 1;; w = EXACT ? w + 1 : w < 31 ? 4 * w + 3 : w + 64) {
+            const int plain = min(w, a.k);
+            for (; s < plain; ++s) step(s, std::integral_constant<bool, false>());
+            if (s >= a.k || step(s, std::integral_constant<bool, true>())) break;
+            ++s;
         }
     };
     if constexpr (EXACT) {
