@@ -489,12 +489,31 @@ cudaError_t ensure_dyn_smem(int dev, const void *fn, int bytes) {
 // 3D: whether the TMA-pipelined kernel runs the hierarchical cycles (binary32,
 // automatic pipeline choice, at least 8 subdomains per SM, as in 2D).
 bool want_ppc3(const hj_handle *h, bool classic) {
-    if (classic || !h->k3 || h->d.dim != 3 || h->p.method != HJ_METHOD_HIER || !h->k3->ppc[0]) return false;
+    if (classic || !h->k3 || h->d.dim != 3 || h->p.method != HJ_METHOD_HIER || !h->k3->one.fn[0]) return false;
     if (h->p.pipeline != -1) return false;
     const Tile3Info *t3 = h->k3;
     const long long nsub = (long long)((h->d.nx + t3->tx - 1) / t3->tx) * ((h->d.ny + t3->ty - 1) / t3->ty) *
                            ((h->d.nz + t3->tz - 1) / t3->tz);
     return nsub >= 8LL * h->nsm;
+}
+
+// 3D pipelined kernel: whether 16-wide subdomains run in pairs.  Measured against one
+// per CTA, us for 20 cycles: 512^3 16 x 8 x 8, k = 1 6,400 -> 5,520, k = 4 6,560 -> 6,220;
+// 256^3 1,041 -> 912, 1,066 -> 976; below some 20 subdomains per SM (128^3, k = 4,
+// converging) 5 % slower.  An odd number of subdomains leaves half of the last pair
+// idle: 112 x 300 x 300 718 -> 836, 773 -> 962; 40 x 500 x 500, k = 4 985 -> 1,298; with one
+// subiteration, and no residual, the wider rows outweigh one in 16 (240^3 848 -> 805,
+// 400^3 3,107 -> 2,829).  Cycles bound by their sweeps have more warps with single ones
+// (k = 8, 448^3: 5,897 -> 5,988, 16 x 8 x 4 6,012 -> 6,250; 16 x 8 x 4 converging, k = 4
+// 15,602 -> 15,916).
+bool ppc3_pairs(const hj_handle *h, bool res) {
+    const Tile3Info *t3 = h->k3;
+    if (!t3->pair.fn[0] || h->p.k > 4) return false;
+    const int sx = (h->d.nx + t3->tx - 1) / t3->tx;
+    const long long nsub = (long long)sx * ((h->d.ny + t3->ty - 1) / t3->ty) * ((h->d.nz + t3->tz - 1) / t3->tz);
+    if (nsub < 20LL * h->nsm) return false;
+    if (sx % 2) return h->p.k == 1 && !res && sx >= 15;
+    return h->p.k == 1 || !res || t3->tz > 4;
 }
 
 // Whether the TMA-pipelined kernel runs this plan's cycles.
@@ -565,15 +584,16 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
             // the next launch over three rotating iterate buffers
             if (res && !b2) return seterr(HJ_ERR_CUDA, "internal: pipelined residual runs need a third iterate buffer");
             const Tile3Info *t3 = h->k3;
-            PpcKernel fn = t3->ppc[res];
-            const int smem = t3->ppc_smem;
+            const Ppc3Info &pc = ppc3_pairs(h, res) ? t3->pair : t3->one;
+            PpcKernel fn = pc.fn[res];
+            const int smem = pc.smem;
             CKR(ensure_dyn_smem(h->dev, (const void *)fn, smem));
             int occ = 0;
-            CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 32 * t3->ppc_ns, smem));
+            CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 32 * pc.ns, smem));
             if (occ < 1) return seterr(HJ_ERR_UNSUPPORTED, "3D pipelined kernel does not fit on an SM");
             if (h->p.ctas_per_sm > 0) occ = std::min(occ, h->p.ctas_per_sm);
-            else if (t3->ppc_cps > 0) occ = std::min(occ, t3->ppc_cps);
-            const int cx = t3->tx * t3->ppc_ns;   // columns a CTA takes at a time
+            else if (pc.cps > 0) occ = std::min(occ, pc.cps);
+            const int cx = t3->tx * pc.ns;   // columns a CTA takes at a time
             const int tiles_x = (nx + cx - 1) / cx, tiles_y = (ny + t3->ty - 1) / t3->ty;
             const int ntiles = tiles_x * tiles_y * ((h->d.nz + t3->tz - 1) / t3->tz);
             const int grid = std::min(ntiles, occ * h->nsm);
@@ -606,7 +626,7 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
             pl->pfn = fn;
             pl->smem = smem;
             pl->grid = dim3(grid);
-            pl->block = dim3(32 * t3->ppc_ns);
+            pl->block = dim3(32 * pc.ns);
             return HJ_OK;
         }
         if (classic) {

@@ -920,21 +920,23 @@ __global__ void __launch_bounds__(256) classic3d_kernel(const CycArgs a) {
      {hj::hier3d_kernel<S, T, LX, RY, RZ, NW, EX, false>, hj::hier3d_kernel<S, T, LX, RY, RZ, NW, EX, true>}, \
      {hj::hier3d_pf_kernel<S, T, LX, RY, RZ, NW, EX, false>,                                         \
       hj::hier3d_pf_kernel<S, T, LX, RY, RZ, NW, EX, true>},                                         \
-     (int)((NW) * hj::Pf3Layout<T, LX, RY, RZ>::PER_WARP * sizeof(T)), {nullptr, nullptr}, 0, 0, 1}
+     (int)((NW) * hj::Pf3Layout<T, LX, RY, RZ>::PER_WARP * sizeof(T)), {}, {}}
 
 // binary32 entry of the same TX x TY x TZ shape: the two-column kernel, whose
 // LX / 2 lanes span x with RY / 2 rows per lane group, the one-column
-// prefetching kernel, and the TMA-pipelined two-column kernel with its
-// subdomains per CTA (NS) and its resident CTAs per SM (CPS, measured per shape: more copies in flight slowed
-// the 16-wide boxes sharply)
-#define HJ_K3D_F32(LX, RY, RZ, NW, NS, CPS)                                                              \
+// prefetching kernel, and the TMA-pipelined two-column kernel with one subdomain per
+// CTA at CPS resident CTAs per SM (measured per shape: more copies in flight slowed
+// the 16-wide boxes sharply) and in PAIRs at full residency (Ppc3Layout)
+#define HJ_PPC3(LX, RY, RZ, NS, CPS)                                                                     \
+    {{hj::ppc3d_kernel<(LX) / 2, (RY) / 2, RZ, NS, false>, hj::ppc3d_kernel<(LX) / 2, (RY) / 2, RZ, NS, true>}, \
+     hj::Ppc3Layout<(LX) / 2, (RY) / 2, RZ, NS>::SMEM, (CPS), (NS)}
+#define HJ_K3D_F32(LX, RY, RZ, NW, CPS, PAIR)                                                           \
     {(LX), (32 / (LX)) * (RY), (RZ), 32 * (NW), (NW),                                               \
      {hj::hier3d_pk_kernel<(LX) / 2, (RY) / 2, RZ, NW, false>, hj::hier3d_pk_kernel<(LX) / 2, (RY) / 2, RZ, NW, true>}, \
      {hj::hier3d_pf_kernel<float, float, LX, RY, RZ, NW, false, false>,                              \
       hj::hier3d_pf_kernel<float, float, LX, RY, RZ, NW, false, true>},                              \
-     (int)((NW) * hj::Pf3Layout<float, LX, RY, RZ>::PER_WARP * sizeof(float)),                       \
-     {hj::ppc3d_kernel<(LX) / 2, (RY) / 2, RZ, NS, false>, hj::ppc3d_kernel<(LX) / 2, (RY) / 2, RZ, NS, true>}, \
-     hj::Ppc3Layout<(LX) / 2, (RY) / 2, RZ, NS>::SMEM, (CPS), (NS)}
+      (int)((NW) * hj::Pf3Layout<float, LX, RY, RZ>::PER_WARP * sizeof(float)),                       \
+     HJ_PPC3(LX, RY, RZ, 1, CPS), PAIR}
 
 // the same without the pipelined kernel (8-wide boxes: 48-byte rows, which
 // the copy engine moves too slowly to gain on the one-warp kernel)
@@ -943,4 +945,4 @@ __global__ void __launch_bounds__(256) classic3d_kernel(const CycArgs a) {
      {hj::hier3d_pk_kernel<(LX) / 2, (RY) / 2, RZ, NW, false>, hj::hier3d_pk_kernel<(LX) / 2, (RY) / 2, RZ, NW, true>}, \
      {hj::hier3d_pf_kernel<float, float, LX, RY, RZ, NW, false, false>,                              \
       hj::hier3d_pf_kernel<float, float, LX, RY, RZ, NW, false, true>},                              \
-     (int)((NW) * hj::Pf3Layout<float, LX, RY, RZ>::PER_WARP * sizeof(float)), {nullptr, nullptr}, 0, 0, 1}
+     (int)((NW) * hj::Pf3Layout<float, LX, RY, RZ>::PER_WARP * sizeof(float)), {}, {}}

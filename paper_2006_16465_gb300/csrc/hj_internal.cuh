@@ -455,16 +455,20 @@ const VcKernelInfo *vc_kernels_f64();
 const VcKernelInfo *vc_kernels_f32();
 
 // 3D seven-point kernels: one warp per TX x TY x TZ subdomain, NW subdomains
+// 3D TMA-pipelined kernel (fn null where not built)
+struct Ppc3Info {
+    PpcKernel fn[2];   // [res]
+    int smem;          // dynamic shared memory
+    int cps;           // its resident CTAs per SM unless the caller sets ctas_per_sm (0: as many as fit)
+    int ns;            // its subdomains along x per CTA (one warp each)
+};
 // per CTA of 32 * NW threads, grid ceil(subdomains / NW) CTAs; fn[res].
 struct Tile3Info {
     int tx, ty, tz, threads, nw;
     CycKernel fn[2];
     CycKernel pf[2];   // prefetching persistent variant: grid <= resident CTAs, dynamic smem pf_smem
     int pf_smem;
-    PpcKernel ppc[2];  // TMA-pipelined variant (binary32; null otherwise): ppc_ns warps per CTA, dynamic smem ppc_smem
-    int ppc_smem;
-    int ppc_cps;       // its resident CTAs per SM unless the caller sets ctas_per_sm (0: as many as fit)
-    int ppc_ns;        // its subdomains along x per CTA (one warp each)
+    Ppc3Info one, pair;   // TMA-pipelined variants (binary32): a subdomain per CTA, two side by side (16-wide ones)
 };
 const Tile3Info *tiles3d_f64(int *n);
 const Tile3Info *tiles3d_f32(int *n);

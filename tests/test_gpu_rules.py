@@ -59,3 +59,29 @@ def test_folds_of_many_ctas_equal_the_pipelined_kernel(prec, tile, n):
            for pl in (0, 1)]
     (a, ua), (b, ub) = res
     assert a["status"] == 0 and a["cycles"] == b["cycles"] and np.array_equal(ua, ub)
+
+
+@pytest.mark.parametrize("shape,tile,k", [((64, 224, 224), (16, 8, 8), 1), ((60, 230, 222), (16, 8, 8), 4), ((250, 130, 110), (16, 8, 8), 4),
+                                           ((33, 300, 230), (16, 8, 4), 2), ((240, 120, 120), (16, 8, 8), 1), ((64, 224, 120), (16, 8, 4), 8)])
+def test_3d_pairs_and_single_subdomains_equal_the_one_warp_kernel(shape, tile, k):
+    """Even and odd numbers of 16-wide subdomains, with and without the residual."""
+    import torch
+    nx, ny, nz = shape
+    import paper_2006_16465_gb300 as hj
+    st = W.poisson3d_uniform(nx, ny, nz, seed=1).st
+    g = torch.Generator(device="cuda")
+    g.manual_seed(4)
+    f = hj.alloc_grid(3, nx, ny, torch.float32, nz=nz)
+    f[1:-1, 1:-1, 1:nx + 1] = torch.rand((nz, ny, nx), generator=g, device="cuda") - 0.5
+    u0 = hj.alloc_grid(3, nx, ny, torch.float32, nz=nz)
+    u0[..., :nx + 2] = torch.rand((nz + 2, ny + 2, nx + 2), generator=g, device="cuda") - 0.5
+    for kw in (dict(fixed_cycles=3), dict(tol=0.0, max_cycles=5)):
+        us = []
+        for pipeline in (-1, 0):
+            s = hj.Solver(st, precision="f32", tile_x=tile[0], tile_y=tile[1], tile_z=tile[2], k=k, pipeline=pipeline, **kw)
+            u = u0.clone()
+            out = s.solve(f, u, check=False)
+            assert out["pipeline_stages"] == (1 if pipeline == -1 else 0)
+            s.close()
+            us.append(u[..., :nx + 2])
+        assert torch.equal(us[0], us[1])
