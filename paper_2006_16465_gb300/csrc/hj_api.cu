@@ -378,10 +378,16 @@ int get_graph(hj_handle *h, void (*fn)(Args), dim3 grid, dim3 block, int smem, c
 }
 
 // Whether the per-point-coefficient cycles run the kernel with four rows a warp
-// (vc2d_rows_kernel: binary32 2D subdomains 32 wide, 4 to 32 rows high).
+// (vc2d_rows_kernel: binary32 2D subdomains 32 wide, 4 to 32 rows high).  Its
+// subiteration is a longer chain (140 against 53 ns on idle SMs), so grids that do not
+// fill the chip keep a thread per point, us for 20 cycles of k = 16 with a thread per
+// point and with rows: 96 x 70, 32 x 8 126, 156; 320 x 300 130, 158; 400 x 350 166, 160;
+// 32 x 32 subdomains (1,024 threads a CTA) 164, 158 already at 96 x 70; k = 64: 400 x 350
+// 249, 281, 500 x 400 332, 284.
 bool vc_rows(const hj_handle *h) {
-    return h->d.coef && h->d.dim == 2 && h->fam_outer == FAM_F32 && h->p.tile_x == 32 && h->p.tile_y % 4 == 0 &&
-           h->p.tile_y <= 32;
+    if (!h->d.coef || h->d.dim != 2 || h->fam_outer != FAM_F32 || h->p.tile_x != 32 || h->p.tile_y % 4 || h->p.tile_y > 32)
+        return false;
+    return h->p.tile_y >= 28 || (long long)h->d.nx * h->d.ny >= (h->p.k <= 16 ? 900LL : 1300LL) * h->nsm;
 }
 
 // Launch plan for one iteration kernel: either the one-CTA-per-tile kernel

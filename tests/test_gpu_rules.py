@@ -85,3 +85,16 @@ def test_3d_pairs_and_single_subdomains_equal_the_one_warp_kernel(shape, tile, k
             s.close()
             us.append(u[..., :nx + 2])
         assert torch.equal(us[0], us[1])
+
+
+@pytest.mark.parametrize("tile", [(32, 4), (32, 12), (32, 24), (32, 32)])
+@pytest.mark.parametrize("n,threads_per_point", [((457, 313), False), ((130, 70), True)])
+def test_varcoef_rows_and_points_match_oracle(tile, n, threads_per_point):
+    """Four rows a warp from 900 points per SM on, a thread per point below."""
+    p = W.variable_coef_problem(2, *n, seed=6, contrast=8.0, screening=20.0)
+    out, u = _solve(p, 2, precision="f32", tile_x=tile[0], tile_y=tile[1], k=3, fixed_cycles=4)
+    rows = not threads_per_point or tile[1] >= 28
+    assert out["tile_threads"] == (8 if rows else 32) * tile[1]
+    assert rel_max(u, oracle.run_fixed(p.st, p.f, p.u0, 4, tile[0], tile[1], 3)) <= 1e-5
+    out, u = _solve(p, 2, precision="f32", tile_x=tile[0], tile_y=tile[1], k=3, tol=0.0, max_cycles=9)
+    assert rel_max(u, oracle.run_fixed(p.st, p.f, p.u0, 9, tile[0], tile[1], 3)) <= 1e-5
