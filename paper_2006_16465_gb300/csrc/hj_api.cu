@@ -555,17 +555,21 @@ bool deferred_run(const hj_handle *h, const TileKernelInfo *ki, const PpcKernelI
 
 
 // Resident CTAs per SM of the 2D pipelined kernel where the caller leaves the
-// choice.  HBM serves the box copies at its full rate up to about 93 KB of them
-// in flight per SM and more slowly beyond (8192 x 8192 binary32, us a cycle, at
-// full residency and at the cap: 32 x 32, 12 -> 10 CTAs: k = 1 136.6 -> 121.6,
-// k = 4 137.6 -> 122.5; 32 x 16, 22 -> 19: 132.5 -> 121, 128.7 -> 121; 64 x 32,
-// 6 -> 5: 131.8 -> 119.4, 130.3 -> 121.6).  Grids that L2 holds (3000 x 2000: no
-// difference at k = 1, 15.1 against 17.2 at k = 4) and cycles bound by their
-// sweeps (k = 5: 138 against 123, k = 6: 126 against 132, k = 16: 224 against
-// 255) want every warp that fits.
+// choice.  HBM serves the box copies of the smaller subdomains at its full rate up to
+// about 93 KB of them in flight per SM and more slowly beyond, once the grid is well
+// beyond L2 and as long as the sweeps are short.  Binary32, us for 90 cycles at full
+// residency and at the cap: 32 x 32 (12 -> 10 CTAs), k = 4: 8192^2 13,725, 12,106, 6000^2
+// 7,188, 6,840, 5000^2 5,113, 5,009, 4096^2 3,460, 3,479, 3400^2 2,477, 2,616; k = 5: 13,243,
+// 12,540, 7,116, 7,176, 5,078, 5,250; 32 x 16 (22 -> 19), k = 4: 8192^2 12,969, 12,425, 5000^2
+// 5,080, 5,102; 64 x 32 (6 -> 5), k = 4: 8192^2 12,822, 12,062, 6000^2 6,930, 6,888, 5000^2
+// 4,909, 5,013, k = 5 slower everywhere; 64 x 64 and 128 x 32 slower everywhere (8192^2,
+// k = 4 12,160, 13,252 and 12,157, 12,930), 32 x 64 too (12,027, 12,395).
 int default_residency(const hj_handle *h, const PpcKernelInfo *pi, int fam, bool sig) {
-    if (fam != FAM_F32 || sig || pi->stages != 1 || h->p.k > 5) return 1 << 20;
-    if (3 * (long long)h->rows * h->d.ld * 4 <= (long long)h->l2_bytes) return 1 << 20;
+    const int all = 1 << 20, pts = pi->tx * pi->ty;
+    if (fam != FAM_F32 || sig || pi->stages != 1 || h->p.k > 5 || pts > 2048) return all;
+    if (pts == 2048 && (h->p.k > 4 || pi->tx != 64)) return all;
+    const long long times_l2 = pts == 2048 ? 3 : h->p.k == 5 ? 4 : 2;
+    if (3 * (long long)h->rows * h->d.ld * 4 <= times_l2 * h->l2_bytes) return all;
     const int flight = 4 * (pi->bwu * (pi->ty + 2) + pi->bwf * pi->ty);   // one CTA's copies, bytes
     return std::max(1, 95 * 1024 / flight);
 }
