@@ -350,6 +350,20 @@ cudaError_t launch_make_dinv_box(const double *sigma, double dconst, long long l
     return cudaGetLastError();
 }
 
+// Whether the 2D residual with constant coefficients runs the row-walking kernel.
+// Measured, us a call of hj_residual (||f|| too, binary64 arrays unless said) with a
+// point per thread and with rows: 256^2 30.5, 32.3; 512^2 42.5, 32.5; 1024^2 54.9, 56.3;
+// 1500^2 67, 80; 2048^2 96, 106; 3000^2 170, 169; 4096^2 290, 269; 6000^2 573, 527; binary32
+// 512^2 42.4, 33.4; 1500^2 69, 81; 4096^2 267, 302; 8192^2 967, 1080; with r32 written (refinement)
+// as fast up to 1024^2 and from 3000^2 on, 2048^2 107, 129.  So: rows from where the
+// point-per-thread form has more than four CTAs per SM to reduce to 1100^2 points, and in
+// binary64 again where HBM bounds it.
+static bool residual_rows(int user_f64, const float *r32, int nx, int ny) {
+    const long long ctas = (long long)((nx + 31) / 32) * ((ny + 7) / 8), pts = (long long)nx * ny;
+    if (ctas <= 4LL * sm_count()) return false;
+    return pts <= 1100LL * 1100 || (user_f64 && !r32 && pts >= 3000LL * 3000);
+}
+
 cudaError_t launch_residual_ex(int dim, int user_f64, const void *f, const void *u, const double *sigma,
                                long long ld, long long ld2, int nx, int ny, double cW, double cE, double cS,
                                double cN, double dconst, int with_fnorm, float *r32, RedArgs red, cudaStream_t s,
@@ -359,7 +373,7 @@ cudaError_t launch_residual_ex(int dim, int user_f64, const void *f, const void 
     a.cW = cW; a.cE = cE; a.cS = cS; a.cN = cN; a.dconst = dconst; a.red = red;
     a.coef = coef; a.cps = cps;
     const dim3 g = aux_grid(dim, nx, ny), b = aux_block(dim);
-    if (dim == 2 && !coef) {
+    if (dim == 2 && !coef && residual_rows(user_f64, r32, nx, ny)) {
         // (never more CTAs than aux_grid: the reduction workspace is sized by it)
         const long long nb = (long long)((nx + 31) / 32) * ((ny + 8 * kResRows - 1) / (8 * kResRows));
         const dim3 g2((unsigned)std::min<long long>(nb, 8LL * sm_count()));

@@ -98,3 +98,19 @@ def test_varcoef_rows_and_points_match_oracle(tile, n, threads_per_point):
     assert rel_max(u, oracle.run_fixed(p.st, p.f, p.u0, 4, tile[0], tile[1], 3)) <= 1e-5
     out, u = _solve(p, 2, precision="f32", tile_x=tile[0], tile_y=tile[1], k=3, tol=0.0, max_cycles=9)
     assert rel_max(u, oracle.run_fixed(p.st, p.f, p.u0, 9, tile[0], tile[1], 3)) <= 1e-5
+
+
+@pytest.mark.parametrize("n", [(300, 200), (700, 500), (1300, 1000)])
+@pytest.mark.parametrize("prec,sigma", [("f64", "field"), ("f64", "none"), ("f32", "field"), ("f32", "none")])
+def test_residual_forms_match_oracle(n, prec, sigma):
+    """A point a thread, rows (between), and a point a thread again: ||f - A u|| to
+    rounding (binary64 arithmetic on the same inputs)."""
+    import torch
+    p = W.random_bc_problem(2, *n, seed=9, sigma_kind=sigma)
+    if prec == "f32":
+        p.f = p.f.astype(np.float32).astype(np.float64)
+        p.u0 = p.u0.astype(np.float32).astype(np.float64)
+    s = gpu_solver(p, precision=prec)
+    a, _ = s.residual(to_dev(p.f, 2, _dt(prec)), to_dev(p.u0, 2, _dt(prec)))
+    s.close()
+    assert a == pytest.approx(oracle.residual(p.st, p.f, p.u0), rel=1e-12)
