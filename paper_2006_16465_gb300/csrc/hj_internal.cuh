@@ -183,7 +183,9 @@ __host__ __device__ __forceinline__ int subdomain_count(int n, int T, int o) {
 // ---------------------------------------------------------------------------
 template <typename S, typename T> __device__ __forceinline__ T ld_s(const S *p) { return (T)__ldg(p); }
 template <> __device__ __forceinline__ float ld_s<__nv_bfloat16, float>(const __nv_bfloat16 *p) {
-    return __bfloat162float(__ldg(p));
+    // (as 16 bits: the header's __ldg of this type is inline assembly, around which a
+    // guard becomes a branch)
+    return __uint_as_float((unsigned)__ldg((const unsigned short *)p) << 16);
 }
 template <typename S, typename T> __device__ __forceinline__ void st_s(S *p, T v) { *p = (S)v; }
 template <> __device__ __forceinline__ void st_s<__nv_bfloat16, float>(__nv_bfloat16 *p, float v) {

@@ -114,3 +114,13 @@ def test_residual_forms_match_oracle(n, prec, sigma):
     a, _ = s.residual(to_dev(p.f, 2, _dt(prec)), to_dev(p.u0, 2, _dt(prec)))
     s.close()
     assert a == pytest.approx(oracle.residual(p.st, p.f, p.u0), rel=1e-12)
+
+
+@pytest.mark.parametrize("n", [(45, 37), (560, 540)])
+def test_bf16_ragged_subdomains_equal_padded_ones(n):
+    """Guarded 16-bit loads at the ragged edge: the engines that stage by copies
+    (zero fill) and by guarded loads give the same corrections."""
+    p = W.random_bc_problem(2, *n, seed=12, sigma_kind="const")
+    kw = dict(precision="bf16corr_ir", tile_x=32, tile_y=32, k=4, tol=1e-6, inner_tol=1e-2, max_outer=6)
+    (a, ua), (b, ub) = _solve(p, 2, persistent=-1, **kw), _solve(p, 2, persistent=1, **kw)
+    assert a["cycles"] == b["cycles"] and np.array_equal(ua, ub)
