@@ -691,7 +691,9 @@ int make_plan(hj_handle *h, const TileKernelInfo *ki, const PpcKernelInfo *pi, i
     if (!want_ppc(h, pi, classic)) {
         geometry(h, ki, classic, &pl->grid, &pl->block);
         pl->fn = (!classic && overlapped(h)) ? ki->ovl[sig][res] : ki->fn[sig][res];
-        if (res && b2 && defer_hier(h, ki, classic)) {
+        const bool defer = res && b2 && defer_hier(h, ki, classic);
+        if (res && !defer && ki->at_end && pl->fn == ki->fn[0][1]) pl->fn = ki->at_end;
+        if (defer) {
             // deferred fold: launch c reads B[c % 3], writes B[(c+1) % 3] and
             // its per-CTA partials to slot c % 2, folded by launch c + 1
             // (the reduction workspace holds two slots of one partial per subdomain)

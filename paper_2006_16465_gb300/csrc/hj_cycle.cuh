@@ -575,9 +575,19 @@ __device__ __forceinline__ float sweeps2d_fold(Tile2D<float, C, R, SIG> &t, cons
         }
     };
     sweep(std::integral_constant<bool, true>());
-    for (int s = 1; s < k; ++s) {
-        exchange();
-        sweep(std::integral_constant<bool, false>());
+    if constexpr (C == 4 && RES) {
+        // (two at a time: 128 x 32 subdomains, 1000 x 960, k = 64 29.5 -> 28.1 us a cycle;
+        // not without the residual: 24.5 -> 26.5)
+#pragma unroll 2
+        for (int s = 1; s < k; ++s) {
+            exchange();
+            sweep(std::integral_constant<bool, false>());
+        }
+    } else {
+        for (int s = 1; s < k; ++s) {
+            exchange();
+            sweep(std::integral_constant<bool, false>());
+        }
     }
     return acc;
 }
@@ -886,20 +896,50 @@ __device__ __forceinline__ void store2d(const Tile2D<T, C, R, SIG> &t, const Cyc
     }
 }
 
-// stop (nullable): set where the run has already ended; read with the staging
-// loads in flight, it ends the CTA before the sweeps (nothing is written).
+// The flags of the CTA's threads or'ed where on (the same for every thread) is set, else
+// this thread's own: a predicated barrier instead of a branch around one.
+__device__ __forceinline__ int barrier_or_if(bool on, int flags) {
+    int r;
+    asm volatile("{\n\t.reg .pred p, q, f;\n\tsetp.ne.s32 p, %1, 0;\n\tsetp.ne.s32 f, %2, 0;\n\tsetp.ne.s32 q, %2, 0;\n\t"
+                 "@p barrier.cta.red.or.pred q, 0, f;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+                 : "=r"(r) : "r"((int)on), "r"(flags) : "memory");
+    return r;
+}
+
+// Whether the run has ended, from this thread's view of the flags.  This launch's
+// fold may be setting them now, so the warps of a CTA may see different answers.  What
+// a launch writes then is not used (three buffers in turn), so they need not agree,
+// and no warp waits for the others' loads here; a warp that has left counts as arrived
+// at the barriers of the others.  In place the array is the result: one answer.
+template <int NW>
+__device__ __forceinline__ int run_ended(const CycArgs &a, int flags) {
+    if constexpr (NW > 1) flags = barrier_or_if(a.uin == a.uout, flags);
+    return __any_sync(FULL, flags);
+}
+
+// Subdomains of two warps that do not overlap keep one answer for the CTA, and stage in
+// front of it in every launch: binary32, 32 x 32, 400 x 380, k = 64 9.7 us a cycle, 10.5
+// with the answers apart (four warps, 200 x 150: 8.3 and 7.8).
+template <int NW, bool OVL>
+constexpr bool kOneAnswer = NW == 2 && !OVL;
+
+// check: stop is set where the run has already ended; read with the staging loads in
+// flight, it ends the warp before the sweeps (nothing is written), and becomes the
+// warp's answer.
 template <typename S, typename T, int C, int R, int NW, int H, bool EXACT, bool SIG, bool RES, bool PART,
           bool OVL = false>
 __device__ __forceinline__ typename std::conditional<EXACT, double, T>::type
 tile2d(const CycArgs &a, const int x0, const int y0, T *xbuf, const Own own = Own{0, 0, 0, 0},
-       const int *stop = nullptr) {
+       const bool check = false, int *stop = nullptr) {
     const int yb = y0 + band_of_lane<R, H>() * R;
     const Coef<T> kc = make_coef<T>(a);
     Tile2D<T, C, R, SIG> t;
     stage2d_global<S, T, C, R, H, EXACT, SIG, PART>(t, a, kc, x0, yb);
-    if (stop) {
-        // one answer for the whole CTA: this launch's fold may be setting the flag now
-        if (NW == 1 ? __any_sync(FULL, *stop) : __syncthreads_or(*stop)) return 0;
+    if constexpr (kOneAnswer<NW, OVL>) {
+        if (check && __syncthreads_or(*stop)) return 0;
+    } else if (check) {
+        *stop = run_ended<NW>(a, *stop);
+        if (*stop) return 0;
     }
     auto acc = sweeps2d<T, C, R, NW, H, EXACT, SIG, RES, PART, OVL>(t, kc, a.k, x0, yb, a.nx, a.ny, xbuf, own, a.dbg);
     store2d<S, T, C, R, H, SIG, PART, OVL>(t, a, x0, yb, own);
@@ -950,8 +990,10 @@ __global__ void __launch_bounds__(32 * NW) hier2d_kernel(const CycArgs a) {
             by = tile / a.jx;
             bx = tile - by * a.jx;
             stop = (ctl->done >= 0) | ctl->fold_only[a.parity];
-        } else {
+        } else if constexpr (kOneAnswer<NW, OVL>) {
             stop = ctl->done >= 0;
+        } else if (ctl->done >= 0) {
+            return;   // (set by an earlier launch)
         }
     }
     constexpr int TX = 32 * C / H, TY = R * NW * H;
@@ -968,13 +1010,17 @@ __global__ void __launch_bounds__(32 * NW) hier2d_kernel(const CycArgs a) {
     }
     const bool full = (x0 + TX - 1 <= a.nx) && (y0 + TY - 1 <= a.ny);
     typename std::conditional<EXACT, double, T>::type acc;
-    if (full) acc = tile2d<S, T, C, R, NW, H, EXACT, SIG, RES, false, OVL>(a, x0, y0, xbuf, own, RES ? &stop : nullptr);
-    else acc = tile2d<S, T, C, R, NW, H, EXACT, SIG, RES, true, OVL>(a, x0, y0, xbuf, own, RES ? &stop : nullptr);
+    const bool check = RES && (kOneAnswer<NW, OVL> || a.part_w);
+    if (full) acc = tile2d<S, T, C, R, NW, H, EXACT, SIG, RES, false, OVL>(a, x0, y0, xbuf, own, check, &stop);
+    else acc = tile2d<S, T, C, R, NW, H, EXACT, SIG, RES, true, OVL>(a, x0, y0, xbuf, own, check, &stop);
     if constexpr (RES) {
-        // (a stopped CTA's partial and reduction share are never read: the run's
-        // answer stands, and the next solve resets the control block)
-        if (a.part_w) write_cta_partial<NW>(a.part_w + tile, acc);
-        else if (!stop) reduce_grid_acc(a.red, acc);
+        if (a.part_w) {
+            // (a stopped CTA's partial is never read: the run's answer stands, and the
+            // next solve resets the control block)
+            if (kOneAnswer<NW, OVL> || !stop) write_cta_partial<NW>(a.part_w + tile, acc);
+        } else if (!kOneAnswer<NW, OVL> || !stop) {
+            reduce_grid_acc(a.red, acc);
+        }
     }
 }
 
@@ -1068,7 +1114,7 @@ struct Xchg1D {
 template <typename S, typename T, int C, int WPT, bool EXACT, bool SIG, bool RES, bool PART, bool OVL = false>
 __device__ __forceinline__ typename std::conditional<EXACT, double, T>::type
 tile1d(const CycArgs &a, const int x0, const int row, Xchg1D<T, WPT> &xb, const int own_lo = 0, const int own_hi = 0,
-       const int *stop = nullptr) {
+       const bool check = false, int *stop = nullptr) {
     constexpr int TX = 32 * C * WPT;
     const int lane = threadIdx.x & 31, q = (threadIdx.x >> 5) % WPT;
     const int xl = x0 + q * 32 * C + lane * C;
@@ -1101,10 +1147,10 @@ tile1d(const CycArgs &a, const int x0, const int row, Xchg1D<T, WPT> &xb, const 
     const int hcol = wl ? x0 - 1 : x0 + TX;
     const bool hok = (wl || el) && (!PART || hcol <= nx + 1) && HJ_IN(a.dbg, rb + hcol, grid_elems1d(a), 32);
     const T hx = hok ? ld_s<S, T>(uin + rb + hcol) : (T)0;
-    // the run has already ended (read beside the loads above, one answer per CTA
-    // where warps meet at barriers)
-    if (stop) {
-        if (WPT == 1 ? __any_sync(FULL, *stop) : __syncthreads_or(*stop)) return 0;
+    // the run has already ended (read beside the loads above)
+    if (check) {
+        *stop = run_ended<WPT>(a, *stop);
+        if (*stop) return 0;
     }
 
     typedef typename std::conditional<EXACT, double, T>::type Acc;
@@ -1179,8 +1225,24 @@ tile1d(const CycArgs &a, const int x0, const int row, Xchg1D<T, WPT> &xb, const 
     return acc;
 }
 
-template <typename S, typename T, int C, int WPT, int WPB, bool EXACT, bool SIG, bool RES, bool OVL = false>
-__global__ void __launch_bounds__(32 * WPT * WPB) hier1d_kernel(const CycArgs a) {
+// Registers of the binary32 cycles with the residual: those of the cycles without the
+// run-ended flags (32, or 40 with eight points a lane), for too few warps in flight
+// otherwise where the lines are beyond L2 (2000 points x 8000 lines in 128-point
+// subdomains, k = 16: 77 us a cycle, 87 with 40 registers).  From four points a lane on
+// only where the run reduces at a launch's end (ATEND); grids that fold in the next
+// launch are small enough (256 points x 8000 lines in 256-point subdomains 21.6 us,
+// 27.6 with 40 registers).  0: the compiler's choice.
+template <typename T, int C, int NW, bool PLAIN, bool ATEND>
+constexpr int hier1d_min_ctas() {
+    if (!std::is_same<T, float>::value || !PLAIN) return 0;
+    return C <= 2 || (ATEND && C <= 4) ? 64 / NW : ATEND ? 48 / NW : 0;
+}
+
+template <typename S, typename T, int C, int WPT, int WPB, bool EXACT, bool SIG, bool RES, bool OVL = false,
+          bool ATEND = false>
+__global__ void __launch_bounds__(32 * WPT * WPB,
+                                  hier1d_min_ctas<T, C, WPT * WPB, RES && !SIG && !OVL, ATEND>())
+    hier1d_kernel(const CycArgs a) {
     static_assert(WPT == 1 || WPB == 1, "several subdomains per CTA only with one warp each");
     int bx = blockIdx.x, row = blockIdx.y, stop = 0, blk = 0;
     if constexpr (RES) {
@@ -1196,8 +1258,8 @@ __global__ void __launch_bounds__(32 * WPT * WPB) hier1d_kernel(const CycArgs a)
             row = blk / gx;
             bx = blk - row * gx;
             stop = (ctl->done >= 0) | ctl->fold_only[a.parity];
-        } else {
-            stop = ctl->done >= 0;
+        } else if (ctl->done >= 0) {
+            return;   // (set by an earlier launch)
         }
     }
     constexpr int TX = 32 * C * WPT;
@@ -1217,14 +1279,19 @@ __global__ void __launch_bounds__(32 * WPT * WPB) hier1d_kernel(const CycArgs a)
     typename std::conditional<EXACT, double, T>::type acc = 0;
     // with WPT > 1, the subdomain is uniform across the CTA and the whole CTA
     // takes the same branch; with WPB > 1 the branches hold no barrier
-    const int *sp = RES ? &stop : nullptr;
+    const bool check = RES && a.part_w;
     if (here) {
-        if (x0 + TX - 1 <= a.nx) acc = tile1d<S, T, C, WPT, EXACT, SIG, RES, false, OVL>(a, x0, row, xb, lo, hi, sp);
-        else acc = tile1d<S, T, C, WPT, EXACT, SIG, RES, true, OVL>(a, x0, row, xb, lo, hi, sp);
+        if (x0 + TX - 1 <= a.nx) acc = tile1d<S, T, C, WPT, EXACT, SIG, RES, false, OVL>(a, x0, row, xb, lo, hi, check, &stop);
+        else acc = tile1d<S, T, C, WPT, EXACT, SIG, RES, true, OVL>(a, x0, row, xb, lo, hi, check, &stop);
+    } else if (check) {
+        stop = __any_sync(FULL, stop);
     }
     if constexpr (RES) {
-        if (a.part_w) write_cta_partial<WPT * WPB>(a.part_w + blk, acc);
-        else if (!stop) reduce_grid_acc(a.red, acc);
+        if (a.part_w) {
+            if (!stop) write_cta_partial<WPT * WPB>(a.part_w + blk, acc);
+        } else {
+            reduce_grid_acc(a.red, acc);
+        }
     }
 }
 
@@ -1646,7 +1713,8 @@ __global__ void __launch_bounds__(256) classic1d_kernel(const CycArgs a) {
      {{hj::hier1d_kernel<S, T, C, WPT, WPB, EX, false, false, true>,                                 \
        hj::hier1d_kernel<S, T, C, WPT, WPB, EX, false, true, true>},                                 \
       {hj::hier1d_kernel<S, T, C, WPT, WPB, EX, true, false, true>,                                  \
-       hj::hier1d_kernel<S, T, C, WPT, WPB, EX, true, true, true>}}}
+       hj::hier1d_kernel<S, T, C, WPT, WPB, EX, true, true, true>}},                                 \
+     1, hj::hier1d_kernel<S, T, C, WPT, WPB, EX, false, true, false, !(EX) && (C) >= 4>}
 #define HJ_KC2D(S, T, EX)                                                                             \
     {2, 32, 8, 256, 1,                                                                               \
      {{hj::classic2d_kernel<S, T, EX, false, false>, hj::classic2d_kernel<S, T, EX, false, true>},   \

@@ -443,6 +443,7 @@ struct TileKernelInfo {
     CycKernel fn[2][2]; // [sig][res]
     CycKernel ovl[2][2];// [sig][res] overlapping subdomains (null for classic kernels)
     int cluster = 1;    // CTAs per subdomain (a cluster along x)
+    CycKernel at_end = nullptr;  // 1D: fn[0][1] for runs that reduce at a launch's end
 };
 
 // Variable-coefficient kernels: [dim - 1][res], one thread per point, dynamic
