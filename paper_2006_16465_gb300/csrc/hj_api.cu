@@ -177,9 +177,10 @@ const TileKernelInfo *find_tile(int fam, int dim, int tx, int ty, int threads = 
 // overlapping points and k = 64 (484) 10.2, 10.8, 11.2.  Binary64 (its first
 // variant has four warps, one per sub-partition's FP64 pipe) gains the waits of
 // one warp filled by another (and clusters of CTAs below that, cluster_choice):
-// k = 16 with 2, 4, 8 warps: 256 x 256 63, 40, 36;
+// k = 16 with 2, 4, 8 warps, every product on the FP64 pipe: 256 x 256 63, 40, 36;
 // 500 x 300 (160) 87, 77, 75; 900 x 800 (725) 194, 177, 175; 3001 x 2003
-// (5,922) 1352, 1315, 1315.  In-place runs choose for the persistent engine instead
+// (5,922) 1352, 1315, 1315.  (With products by constants on the integer pipes eight
+// warps are ahead beyond the line drawn here too: 900 x 800 137 with four, 123.)  In-place runs choose for the persistent engine instead
 // (in_place_threads).
 int default_threads(int fam, const hj_desc &d, const hj_params &p, int nsm) {
     if (d.dim != 2 || p.method != HJ_METHOD_HIER || d.coef || p.persistent == 1 || p.pipeline == 1 || p.in_place) return 0;
@@ -788,8 +789,9 @@ struct RunOut {
     void *buf;          // the buffer that holds iterate c
 };
 
-// Where a converging run keeps its third iterate buffer (allocated on first use:
-// the deferred residual fold needs it).
+// Where a converging run keeps its third iterate buffer (allocated on first use: the
+// deferred residual fold needs it, in the pipelined kernels and up to defer_max_blocks
+// CTAs in the one-CTA-per-subdomain ones).
 struct ThirdBuffer {
     void **slot;
     size_t bytes;

@@ -123,10 +123,9 @@ __global__ void __launch_bounds__(256) residual_kernel(const AuxArgs a) {
 // The same with constant neighbour coefficients in 2D, a lane walking R rows of
 // its column: every value is loaded and converted to binary64 once, vertical
 // neighbours stay in registers, horizontal ones come by shuffle.  Bound by the
-// FP64 pipe (five multiply-adds a point, one for each norm); the point-per-thread
-// form above waited for five loads and five conversions a point beside them.
-// With ||f||, 8192 x 8192 binary32: 1.66 -> 1.26 ms (the pipe alone: 0.89);
-// 4096 x 4096 binary64 0.297 -> 0.274 ms.
+// FP64 pipe (five multiply-adds a point, one for each norm) and, with a warp's eight
+// rows one after the other, by too few loads in flight: both forms are measured at
+// residual_rows, which chooses.
 constexpr int kResRows = 8;
 template <typename T, bool WITH_F>
 __global__ void __launch_bounds__(256) residual2d_kernel(const AuxArgs a) {

@@ -241,8 +241,9 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
     // (late: the checks of the cycle before are queue entries too)
     // one-warp CTAs: two per scheduler.  At the full twelve per SM their copies, all
     // issued behind the same barrier, wait 18 us for the first box; ten leave the
-    // schedulers uneven (64 problems of sides 64 to 512, all active: 12, 10, 8, 7, 6
-    // CTAs per SM 41.0, 41.1, 37.1, 38.9, 41.7 us a cycle)
+    // schedulers uneven (64 problems of sides 64 to 512, 32 x 32 subdomains, all active:
+    // 12, 10, 8, 7, 6 CTAs per SM 41.0, 41.1, 37.1, 38.9, 41.7 us a cycle; other heights
+    // are held to the same count and not measured apart)
     if (late && !sig && threads == 32) cap = std::min(cap, 8 * h->nsm);
     L->grid = (int)std::min<long long>(nitems + (late ? nprob : 0), cap);
     L->threads = threads;

@@ -1432,8 +1432,8 @@ __global__ void __launch_bounds__(1024, 2) vc_kernel(const CycArgs a) {
 // 1/d), and the thread-per-point one above kept too little in flight to fill it:
 // at 32 x 32 two CTAs of 1024 threads are all an SM holds, eight loads a thread,
 // and both phases of a CTA (load, sweep) wait at every barrier.  Here a CTA has
-// 256 threads of 28 to 32 independent loads each and five or more CTAs share an
-// SM.  Same sums in the same order, so the iterates are equal bit for bit.
+// 256 threads of 28 to 32 independent loads each and four CTAs share an SM (by
+// registers).  Same sums in the same order, so the iterates are equal bit for bit.
 // Measured at 4096 x 4096, 32 x 32, k = 4: 145.8 -> 94.9 us a cycle (5.7 TB/s), k = 1
 // 130.5 -> 84.3; 32 x 8, k = 4 117.4 -> 91.0.
 template <bool RES>

@@ -11,13 +11,15 @@
 //   * mg_smooth_kernel: one weighted hierarchical cycle, a thread per point of
 //     up to four rows, the subdomain plus halo in two shared-memory
 //     containers, k damped Jacobi subiterations u' = u + omega (jac - u)
-//     with the halo frozen;
+//     with the halo frozen (binary32 subdomains 32 wide and a multiple of four
+//     high: mg_smooth_rows_kernel, four rows a warp in registers);
 //   * mg_restrict_kernel (binary32), mg_restrict_tile_kernel (binary64): the fine
 //     residual f - A u at the nine fine points around each coarse point,
 //     full-weighted into the coarse right-hand side (fused, no residual array),
 //     and the coarse correction set to zero;
 //   * mg_prolong_kernel: u + bilinear interpolation of the coarse correction,
-//     one thread per coarse cell writing the 2 x 2 fine points inside it.
+//     one thread per coarse cell writing the 2 x 2 fine points from its first
+//     coarse point on.
 // The graph also holds the residual norm of the level-0 iterate and its copy
 // to pinned host memory, so a V-cycle costs one graph launch and one wait.
 //
@@ -647,10 +649,11 @@ void launch_restrict(const hj_handle *h, const MgXferArgs &x, int ncx, int ncy, 
 // Launch count: on levels of a few hundred thousand points or fewer a launch
 // costs its fixed latency (a few microseconds) whatever its size, so there the
 // transfers are folded into the launches next to them where the result is the
-// same: the restriction into the coarse level's first smoothing (which forms
+// same: in binary32 the restriction into the coarse level's first smoothing (which forms
 // the coarse RHS for its subdomain while staging, stores it for the level's
 // later launches, and starts from a zero correction, as the restriction sets
-// it) and the prolongation into the fine level's first post-smoothing (which
+// it; in binary64, bound by the sums that the subdomains' halos would repeat, it stays a
+// launch) and the prolongation into the fine level's first post-smoothing (which
 // stages u + P e for its subdomain and halo).  On larger levels the separate
 // transfer kernels stay: they form each value once with coalesced accesses,
 // where a smoothing launch would recompute the halo's.  The coarsest level's
