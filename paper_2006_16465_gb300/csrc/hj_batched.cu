@@ -54,23 +54,21 @@ int ensure_scratch(hj_handle *h, size_t bytes) {
 
 // TMA-staged persistent kernels run unless pipeline = 0 (2D only).
 bool persist_uses_tma(const hj_handle *h, const PersistKernelInfo *ki, bool sig) {
-    return h->p.pipeline != 0 && ki && ki->dim == 2 && ki->tma_fn[sig] && ki->tma_one[sig];
+    return h->p.pipeline != 0 && ki && ki->dim == 2 && ki->tma_one[sig];
 }
 
 namespace {
 int capacity_of(hj_handle *h, const PersistKernelInfo *ki, bool sig, bool tma, int *ctas) {
-    int occ = 0, occ1 = 0;
-    if (tma) {
-        const int smem = ki->tma_smem[sig];
-        for (PersistKernel fn : {ki->tma_fn[sig], ki->tma_one[sig]})
-            CKR(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ki->tma_fn[sig], ki->threads, smem));
-        CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, ki->tma_one[sig], ki->threads, smem));
-    } else {
-        CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ki->fn[sig], ki->threads, 0));
-        CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, ki->one[sig], ki->threads, 0));
+    int least = 1 << 20;
+    for (PersistKernel fn : {tma ? ki->tma_fn[sig] : ki->fn[sig], tma ? ki->tma_one[sig] : ki->one[sig]}) {
+        if (!fn) continue;
+        const int smem = tma ? ki->tma_smem[sig] : 0;
+        if (tma) CKR(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        int occ = 0;
+        CKR(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, ki->threads, smem));
+        least = std::min(least, occ);
     }
-    *ctas = std::min(occ, occ1) * h->nsm;
+    *ctas = least * h->nsm;
     return HJ_OK;
 }
 }  // namespace
@@ -129,7 +127,7 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
         }
     }
     // the kernel of many problems decides one cycle late, over three buffers
-    bool late = tma;
+    bool late = tma && ki->tma_fn[sig];
     for (auto &p : probs) late = late && p.third;
     if (nprob > 1 && !late) tma = false;   // without third buffers: plain staging, two barriers
     long long nitems = 0, max_iters = 1;
@@ -256,6 +254,7 @@ int persist_setup(hj_handle *h, const PersistKernelInfo *ki, bool sig, std::vect
             : late ? (const void *)ki->tma_fn[sig]
             : tma ? (const void *)ki->tma_one[sig]
             : nprob == 1 ? (const void *)ki->one[sig] : (const void *)ki->fn[sig];
+    if (!L->fn) return seterr(HJ_ERR_UNSUPPORTED, "no persistent kernel of many problems for this precision");
     L->hb = hb;
     L->db = db;
     L->o_state = o_state;

@@ -545,7 +545,7 @@ typedef void (*PersistKernel)(PersistArgs);
 
 struct PersistKernelInfo {
     int dim, tx, ty, threads, tiles_per_cta;
-    PersistKernel fn[2];      // [sig]  many problems, two barriers per cycle
+    PersistKernel fn[2];      // [sig]  many problems, two barriers per cycle (2D binary64: null, as tma_fn)
     PersistKernel one[2];     // [sig]  one problem, one barrier per cycle
     // TMA-staged variants (2D; null otherwise) and their dynamic shared memory
     PersistKernel tma_fn[2], tma_one[2];

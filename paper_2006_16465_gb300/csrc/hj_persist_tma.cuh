@@ -440,14 +440,21 @@ __global__ void __launch_bounds__(32 * NW, (NW == 4 && SIG) ? 3 : 0) persist2d_b
     }
 }
 
+// The kernels of many problems: batches run binary32 arithmetic only (null in binary64).
+template <typename S, typename T, int C, int R, int NW, int H, bool EXACT, bool SIG, bool TMA>
+constexpr PersistKernel many_kernel() {
+    if constexpr (std::is_same<T, double>::value) return nullptr;
+    else if constexpr (TMA) return persist2d_batch_kernel<S, T, C, R, NW, H, EXACT, SIG>;
+    else return persist2d_kernel<S, T, C, R, NW, H, EXACT, SIG>;
+}
+
 }  // namespace hj
 
 #define HJ_KP2D(S, T, C, R, NW, H, EX)                                                                    \
     {2, 32 * (C) / (H), (R) * (NW) * (H), 32 * (NW), 1,                                                  \
-     {hj::persist2d_kernel<S, T, C, R, NW, H, EX, false>, hj::persist2d_kernel<S, T, C, R, NW, H, EX, true>}, \
+     {hj::many_kernel<S, T, C, R, NW, H, EX, false, false>(), hj::many_kernel<S, T, C, R, NW, H, EX, true, false>()}, \
      {hj::persist2d_one_kernel<S, T, C, R, NW, H, EX, false>, hj::persist2d_one_kernel<S, T, C, R, NW, H, EX, true>}, \
-     {hj::persist2d_batch_kernel<S, T, C, R, NW, H, EX, false>,                                         \
-      hj::persist2d_batch_kernel<S, T, C, R, NW, H, EX, true>},                                         \
+     {hj::many_kernel<S, T, C, R, NW, H, EX, false, true>(), hj::many_kernel<S, T, C, R, NW, H, EX, true, true>()}, \
      {hj::persist2d_tma_one_kernel<S, T, C, R, NW, H, EX, false>,                                       \
       hj::persist2d_tma_one_kernel<S, T, C, R, NW, H, EX, true>},                                       \
      {hj::PpcLayout<S, T, C, R, NW, H, false, 1>::SMEM, hj::PpcLayout<S, T, C, R, NW, H, true, 1>::SMEM},  \
