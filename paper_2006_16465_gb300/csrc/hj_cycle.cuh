@@ -917,11 +917,12 @@ __device__ __forceinline__ int run_ended(const CycArgs &a, int flags) {
     return __any_sync(FULL, flags);
 }
 
-// Subdomains of two warps that do not overlap keep one answer for the CTA, and stage in
-// front of it in every launch: binary32, 32 x 32, 400 x 380, k = 64 9.7 us a cycle, 10.5
-// with the answers apart (four warps, 200 x 150: 8.3 and 7.8).
+// Subdomains of two warps that do not overlap, and overlapping ones of one warp, keep
+// one answer for the CTA and stage in front of it in every launch: binary32, 32 x 32,
+// 400 x 380, k = 64 9.7 us a cycle, 10.5 with the answers apart (four warps, 200 x 150:
+// 8.3 and 7.8); 500 x 450, 8 points shared, k = 16 4.65, 4.84.
 template <int NW, bool OVL>
-constexpr bool kOneAnswer = NW == 2 && !OVL;
+constexpr bool kOneAnswer = NW == 2 ? !OVL : NW == 1 && OVL;
 
 // check: stop is set where the run has already ended; read with the staging loads in
 // flight, it ends the warp before the sweeps (nothing is written), and becomes the
@@ -936,7 +937,7 @@ tile2d(const CycArgs &a, const int x0, const int y0, T *xbuf, const Own own = Ow
     Tile2D<T, C, R, SIG> t;
     stage2d_global<S, T, C, R, H, EXACT, SIG, PART>(t, a, kc, x0, yb);
     if constexpr (kOneAnswer<NW, OVL>) {
-        if (check && __syncthreads_or(*stop)) return 0;
+        if (check && (NW == 1 ? __any_sync(FULL, *stop) : __syncthreads_or(*stop))) return 0;
     } else if (check) {
         *stop = run_ended<NW>(a, *stop);
         if (*stop) return 0;
